@@ -103,7 +103,7 @@ struct TuneKey {
 };
 struct TuneRecord {
   TuneKey key;
-  int variant;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored, else warps per target
+  int variant;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored, -5 semi-normal, else warps per target
   float ms;
 };
 
@@ -303,6 +303,28 @@ static cudaError_t launch_single(gmls_ctx* ctx, const StencilJob& j, int variant
   return e;
 }
 
+// The semi-normal-equation kernel on the job's work list; per-group slots for
+// the resident grid, on a small arena a smaller grid (the groups loop over the
+// targets, so any grid is correct).
+static cudaError_t launch_sne(gmls_ctx* ctx, const StencilJob& j, int deg, int kmax, bool neu, int sms) {
+  SneShape sh;
+  cudaError_t e = sne_launch_shape(j.kind, j.dim, deg, j.L, neu, kmax, j.n_tgt, sms, &sh);
+  if (e != cudaSuccess) return e;
+  const size_t per_block = sh.scratch / (size_t)sh.grid;
+  void* scr = ctx->arena.alloc(sh.scratch);
+  while (!scr && sh.grid > 1) {
+    sh.grid = (sh.grid + 1) / 2;
+    sh.scratch = per_block * (size_t)sh.grid;
+    scr = ctx->arena.alloc(sh.scratch);
+  }
+  if (!scr) return cudaErrorMemoryAllocation;
+  StencilJob js = j;
+  js.dscratch = static_cast<unsigned char*>(scr);
+  e = launch_stencils_sne(ctx->launch(), js, deg, sh, neu);
+  ctx->arena.release(scr);  // stream ordered: later work on this stream runs after the kernel
+  return e;
+}
+
 // Uniform neighbour counts and degree: one shape.  Candidates: the register
 // kernel with a warp (variant -1), a half warp (variant -2) or 8 lanes
 // (variant -4; not for Neumann rows, which it has no instantiation for) per
@@ -325,7 +347,20 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
   const bool okdfx = fast_allowed && p->basis == GMLS_BASIS_DIVFREE &&
                      kmax >= gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree) &&
                      dfx_path_available(dim, p->degree, kmax, j.L);
+  // semi-normal-equation kernel (variant -5)
+  const bool oksne = fast_allowed && (p->basis != GMLS_BASIS_DIVFREE || kmax >= gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree)) &&
+                     sne_path_available(p->basis, dim, p->degree, kmax, j.L, false);
+  // It wins every shape it is built for from about 2,000 targets on (2D scalar
+  // m = 4: 44 against 55 us on 3,969 targets, 0.39 against 0.59 ms on 62,500;
+  // 3D scalar m = 3: 58 / 114 us on 4,096; 3D divergence-free m = 3: 0.29 /
+  // 0.55 ms) and the large systems at any size (3D degree 4, 1,000 targets: 0.11
+  // against 0.21 ms scalar, 0.28 against 3.2 ms divergence-free).  Fewer
+  // targets of a small system leave most of its groups without work (2D scalar
+  // m = 3, 1,024 targets: 28 against 22 us): there the autotuner times the
+  // others, unless this context has taken it for the shape before (a shape then
+  // keeps its kernel whatever the number of targets).
   auto launch_fast = [&](const StencilJob& jj, int variant) {
+    if (variant == -5) return launch_sne(ctx, jj, p->degree, kmax, false, sms);
     if (variant == -3) {
       DfxShape sh;
       cudaError_t e = dfx_launch_shape(jj, sms, &sh);
@@ -356,11 +391,15 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
   if (ctx->force_variant != 0) {
     const int v = ctx->force_variant;
     const bool ok = (v == -1 && ok32) || (v == -2 && ok16) || (v == -3 && okdfx) || (v == -4 && ok8) ||
+                    (v == -5 && oksne) ||
                     (v > 0 && variant_fits(v, ld, nmax, refine));
     if (!ok) return fail(ctx, GMLS_EINVAL, "gmls_stencils: the forced kernel variant is not available for this shape");
     choice = v;
   } else if (ctx->force_generic) {
     choice = heuristic_variant(ld, nmax, refine);
+  } else if (oksne && (j.n_tgt >= 2048 || nmax >= 32)) {
+    choice = -5;
+    ctx->tune[key] = choice;
   } else if (it != ctx->tune.end()) {
     choice = it->second;
   } else if (ctx->autotune && !capturing(ctx)) {
@@ -423,7 +462,8 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
     // shape when there is one (a second launch over the list the first one
     // fills), else the shared-memory kernel
     const int mr = choice == -2 ? mr16 : choice == -4 ? mr8 : mr32, hw = choice == -2 ? 16 : choice == -4 ? 8 : 32;
-    const bool neu_fast = choice != -3 && j.neu_items && fast_neu_available(dim, p->degree, mr, j.L, hw);
+    const bool neu_sne = choice == -5 && j.neu_items && sne_path_available(p->basis, dim, p->degree, kmax, j.L, true);
+    const bool neu_fast = neu_sne || (choice > -5 && choice != -3 && j.neu_items && fast_neu_available(dim, p->degree, mr, j.L, hw));
     StencilJob jf = j;
     if (!neu_fast) jf.neu_items = jf.neu_count = nullptr;
     CK(launch_fast(jf, choice), "gmls_stencils fast launch");
@@ -432,19 +472,21 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
       jn.items = jf.neu_items;
       jn.n_items = jf.neu_count;
       jn.neu_items = jn.neu_count = nullptr;
-      CK(launch_stencils_fast(ctx->launch(), jn, mr, hw, sms, true), "gmls_stencils Neumann launch");
+      CK(neu_sne ? launch_sne(ctx, jn, p->degree, kmax, true, sms)
+                 : launch_stencils_fast(ctx->launch(), jn, mr, hw, sms, true), "gmls_stencils Neumann launch");
     }
     // targets the register kernels handed off (tile misfits; Neumann rows
     // without a Neumann instantiation; the factored kernel's well-conditioned
-    // targets that one refinement pass left short of the tolerance): the
+    // targets that one refinement pass left short of the tolerance; the
+    // semi-normal-equation kernel's targets of condition above about 300): the
     // shared-memory FP32 kernel, whose failures join the FP64 redo list
     StencilJob jg = j;
     jg.items = j.gen_items;
     jg.n_items = j.gen_count;
-    // (with uniform neighbour counts only Neumann rows or a tile with fewer
-    // rows than basis functions are handed off)
+    // (with uniform neighbour counts the register kernels hand off only Neumann
+    // rows or a tile with fewer rows than basis functions)
     const int vg = heuristic_variant(ld, nmax, true);
-    if (vg && (p->neumann || ld < nmax || choice == -3))
+    if (vg && (p->neumann || ld < nmax || choice == -3 || choice == -5))
       CK(launch_single(ctx, jg, vg, ld, nmax, true, counter, sms), "gmls_stencils hand-off launch");
   } else
     CK(launch_single(ctx, j, choice, ld, nmax, refine, counter, sms), "gmls_stencils launch");
@@ -715,10 +757,10 @@ gmls_status gmls_set_option(gmls_ctx* ctx, int32_t option, int64_t value) {
       return GMLS_OK;
     case GMLS_OPT_AUTOTUNE: ctx->autotune = value != 0; return GMLS_OK;
     case GMLS_OPT_FORCE_VARIANT:
-      if (value != 0 && value != -1 && value != -2 && value != -3 && value != -4 &&
+      if (value != 0 && value != -1 && value != -2 && value != -3 && value != -4 && value != -5 &&
           !(value > 0 && value < 24 && (v_warps((int)value) == 1 || v_warps((int)value) == 2 ||
                                         v_warps((int)value) == 4)))
-        return fail(ctx, GMLS_EINVAL, "gmls_set_option: variant must be 0, -1 .. -4 or G + 8 * P (G 1, 2, 4; P 0, 1, 2)");
+        return fail(ctx, GMLS_EINVAL, "gmls_set_option: variant must be 0, -1 .. -5 or G + 8 * P (G 1, 2, 4; P 0, 1, 2)");
       ctx->force_variant = (int)value;
       return GMLS_OK;
     case GMLS_OPT_POISON:

@@ -139,6 +139,7 @@ struct StencilJob {
   // work list: items[0..*n_items) are target ordinals; NULL items = all
   const int32_t* items;
   const int32_t* n_items;
+  const int32_t* item_range;  // semi-normal-equation kernel: [begin, end) of items (NULL: items[0..*n_items))
   // basis
   int kind;                // GMLS_BASIS_*
   int degree;
@@ -243,6 +244,19 @@ struct DfxShape {
 cudaError_t dfx_launch_shape(const StencilJob& j, int sms, DfxShape* s);
 // global scratch of a launch over n_tgt targets (0 if the shape is not instantiated)
 size_t dfx_scratch_bytes(int dim, int deg, int64_t n_tgt, int sms);
+// semi-normal-equation kernel (sne.cu): is (basis, dim, degree, L) instantiated
+// for lists of at most kmax neighbours, and its launch; scratch as for the
+// factored kernel
+bool sne_path_available(int kind, int dim, int deg, int kmax, int L, bool neu);
+struct SneShape {
+  int grid, warps;  // blocks, warps per block
+  int kp;           // neighbour capacity
+  size_t smem;      // shared bytes per block
+  size_t scratch;   // global bytes the launch needs in StencilJob::dscratch
+};
+cudaError_t sne_launch_shape(int kind, int dim, int deg, int L, bool neu, int kmax, int64_t n_tgt, int sms,
+                             SneShape* s);
+cudaError_t launch_stencils_sne(const Launch& L, const StencilJob& j, int deg, const SneShape& s, bool neu);
 cudaError_t launch_stencils_dfx(const Launch& L, const StencilJob& j, const DfxShape& s);
 
 // -------------------------------------------------------------------- CSR
