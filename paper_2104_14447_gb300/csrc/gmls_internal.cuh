@@ -208,7 +208,7 @@ struct BucketJob {
   int n_classes;
   int class_rows[16];
   int nb;                       // n_classes * 4 + 1 (the last: too large)
-  int gpb[kMaxBuckets];         // targets per block task
+  int gpb[kMaxBuckets];         // targets per block task (0: the bucket has a launch of its own)
   int32_t* counts;
   int32_t* fill;
   int32_t* bucket_of;
