@@ -1596,9 +1596,11 @@ gmls_status gmls_csr_spmv(gmls_ctx* ctx, int64_t n_rows, const int64_t* row_ptr,
 // ------------------------------------------------------------------- GMRES
 // Restarted GMRES(m) with right Jacobi preconditioning, A D^-1 y = b,
 // x = D^-1 y (D = diag A, 1 where that is zero).  Arnoldi with classical
-// Gram-Schmidt applied twice; the Hessenberg column and the new norm come to
-// the host once per iteration, where Givens rotations update the residual
-// estimate.  The true residual is recomputed at every restart and at the end.
+// Gram-Schmidt applied twice; the Hessenberg columns, their Givens rotations and
+// the residual estimate stay on the device.  The host queues a chunk of
+// iterations and then reads whether the cycle is done; the triangular solve at
+// its end runs on the host.  The true residual is recomputed at every restart
+// and at the end.
 gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const int32_t* col, const double* val,
                        const double* b, double* x, const gmls_gmres_params* p, int32_t* iters, double* rel_residual) {
   if (!ctx) return GMLS_EINVAL;
@@ -1611,17 +1613,19 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
   if (capturing(ctx)) return fail(ctx, GMLS_EBUSY, "gmls_gmres reads the device every iteration: not during capture");
   CK(cudaSetDevice(ctx->device), "gmls_gmres");
   const int m = p->restart;
+  constexpr int kGmresChunk = 8;  // iterations queued before the host looks at done
   double* V = arena_alloc<double>(ctx, (size_t)(m + 1) * n);
   double* z = arena_alloc<double>(ctx, n);
   double* dinv = arena_alloc<double>(ctx, n);
   double* part = arena_alloc<double>(ctx, krylov_partial_elems(m + 2));
-  double* hdev = arena_alloc<double>(ctx, 2 * (m + 2));
+  // H, cs, sn, g, h1, h2, |w|^2 / dot results, y
+  double* hdev = arena_alloc<double>(ctx, (size_t)m * (m + 1) + 2 * m + (m + 1) + 2 * (m + 2) + 2 + m);
   int32_t* long_rows = arena_alloc<int32_t>(ctx, n);
-  int32_t* n_long = arena_alloc<int32_t>(ctx, 1);
+  int32_t* ints = arena_alloc<int32_t>(ctx, 5 + kLongSplitRows);  // n_long, counter, counter, jdone, done, long rows' counters
   double* sp_part = arena_alloc<double>(ctx, csr_spmv_partial_elems());
   const bool rs = p->row_scaling != 0;
   double* rinv = rs ? arena_alloc<double>(ctx, n) : nullptr;
-  void* all[] = {V, z, dinv, part, hdev, long_rows, n_long, sp_part, rinv};
+  void* all[] = {V, z, dinv, part, hdev, long_rows, ints, sp_part, rinv};
   auto release = [&]() {
     for (void* q : all) ctx->arena.release(q);
   };
@@ -1631,14 +1635,26 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
       release();
       return fail(ctx, GMLS_ENOMEM, "gmls_gmres: arena exhausted (the basis needs (restart + 1) n doubles)");
     }
+  GmresState st;
+  st.H = hdev;
+  st.cs = st.H + (size_t)m * (m + 1);
+  st.sn = st.cs + m;
+  st.g = st.sn + m;
+  st.h1 = st.g + (m + 1);
+  st.h2 = st.h1 + (m + 2);
+  st.nrm2 = st.h2 + (m + 2);
+  double* ydev = st.nrm2 + 2;
+  st.jdone = ints + 3;
+  st.done = ints + 4;
+  int32_t *n_long = ints, *counter = ints + 1, *long_counters = ints + 5;
   Launch L = ctx->launch();
-  cudaError_t e = cudaSuccess;
-  auto spmv = [&](const double* in, double* out) {
-    if (e == cudaSuccess) e = launch_csr_spmv(L, n, row_ptr, col, val, in, out, long_rows, n_long, sp_part);
+  cudaError_t e = cudaMemsetAsync(ints, 0, sizeof(int32_t) * (5 + kLongSplitRows), ctx->stream);
+  auto read = [&](void* dst, const void* src, size_t bytes) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, ctx->stream);
   };
   auto dot_host = [&](const double* a, const double* c, double* out_host) {
-    if (e == cudaSuccess) e = krylov_dots(L, n, 1, a, c, part, hdev);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, hdev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = krylov_dots(L, n, 1, a, c, part, st.nrm2, counter, nullptr);
+    read(out_host, st.nrm2, sizeof(double));
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   };
   // with row scaling R (rinv): GMRES on R A D y = R b, x = D y, and the
@@ -1653,12 +1669,24 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
     dot_host(b, b, &bb);
   }
   const double bnorm = std::sqrt(bb);
-  std::vector<double> H((size_t)(m + 1) * m, 0.0), cs(m, 0.0), sn(m, 0.0), g(m + 1, 0.0), hc(2 * (m + 2), 0.0);
-  int total = 0;
+  std::vector<double> H((size_t)(m + 1) * m, 0.0), g(m + 1, 0.0);
+  int total = 0, n_queued = -1;  // long rows (-1: not known yet)
   double rel = 0.0;
+  // A in -> out (scaled by rows if asked): the first call queues the long rows
+  auto spmv = [&](const double* in, double* out, const double* scale, const int32_t* done) {
+    if (e != cudaSuccess) return;
+    if (n_queued >= 0 && n_queued <= kLongSplitRows) {
+      e = launch_csr_spmv_queued(L, n, row_ptr, col, val, in, out, scale, long_rows, n_queued, sp_part, long_counters,
+                                 done);
+      return;
+    }
+    e = launch_csr_spmv(L, n, row_ptr, col, val, in, out, long_rows, n_long, sp_part);
+    if (scale && e == cudaSuccess) e = krylov_scale_in_place(L, n, scale, out);
+  };
   while (e == cudaSuccess) {
     // r = b - A x into V_0
-    spmv(x, V);
+    spmv(x, V, nullptr, nullptr);
+    if (n_queued < 0) read(&n_queued, n_long, sizeof(int32_t));  // complete at dot_host's synchronisation
     if (e == cudaSuccess) e = krylov_residual(L, n, b, V);
     if (rs && e == cudaSuccess) e = krylov_scale_in_place(L, n, rinv, V);
     double rr = 0.0;
@@ -1667,57 +1695,41 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
     rel = bnorm > 0.0 ? beta / bnorm : beta;
     if (e != cudaSuccess || rel <= p->rtol || total >= p->max_iter || !(beta > 0.0)) break;
     if (e == cudaSuccess) e = krylov_scaled_copy(L, n, V, 1.0 / beta, V);
-    std::fill(g.begin(), g.end(), 0.0);
-    g[0] = beta;
-    int jdone = 0;
-    for (int j = 0; j < m && total < p->max_iter && e == cudaSuccess; ++j) {
-      double* vj = V + (size_t)j * n;
-      double* w = V + (size_t)(j + 1) * n;
-      if (e == cudaSuccess) e = krylov_scale(L, n, dinv, vj, z);
-      spmv(z, w);
-      if (rs && e == cudaSuccess) e = krylov_scale_in_place(L, n, rinv, w);
-      // CGS2: h = V^T w, w -= V h, twice; then |w|
-      if (e == cudaSuccess) e = krylov_dots(L, n, j + 1, V, w, part, hdev);
-      if (e == cudaSuccess) e = krylov_axpy(L, n, j + 1, V, hdev, w);
-      if (e == cudaSuccess) e = krylov_dots(L, n, j + 1, V, w, part, hdev + (m + 2));
-      if (e == cudaSuccess) e = krylov_axpy(L, n, j + 1, V, hdev + (m + 2), w);
-      if (e == cudaSuccess) e = krylov_dots(L, n, 1, w, w, part, hdev + (m + 2) + (j + 1));
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(hc.data(), hdev, sizeof(double) * 2 * (m + 2), cudaMemcpyDeviceToHost, ctx->stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-      if (e != cudaSuccess) break;
-      std::vector<double> h(j + 2);
-      for (int i = 0; i <= j; ++i) h[i] = hc[i] + hc[(m + 2) + i];
-      const double hn = std::sqrt(std::max(hc[(m + 2) + (j + 1)], 0.0));
-      h[j + 1] = hn;
-      for (int i = 0; i < j; ++i) {  // previous rotations
-        const double t = cs[i] * h[i] + sn[i] * h[i + 1];
-        h[i + 1] = -sn[i] * h[i] + cs[i] * h[i + 1];
-        h[i] = t;
+    if (e == cudaSuccess) e = krylov_scale(L, n, dinv, V, z);
+    if (e == cudaSuccess) e = krylov_start(L, st, m, beta);
+    const int steps = std::min(m, p->max_iter - total);
+    int32_t flags[2] = {0, 0};  // jdone, done
+    for (int j = 0; j < steps && e == cudaSuccess && !flags[1];) {
+      for (int c = 0; c < kGmresChunk && j < steps; ++c, ++j) {
+        double* w = V + (size_t)(j + 1) * n;
+        spmv(z, w, rinv, st.done);
+        // CGS2: h = V^T w, w -= V h, twice; then |w|
+        if (e == cudaSuccess) e = krylov_dots(L, n, j + 1, V, w, part, st.h1, counter, st.done);
+        if (e == cudaSuccess) e = krylov_axpy(L, n, j + 1, V, st.h1, w, st.done);
+        if (e == cudaSuccess) e = krylov_dots(L, n, j + 1, V, w, part, st.h2, counter, st.done);
+        if (e == cudaSuccess) e = krylov_axpy_norm(L, n, j + 1, V, st.h2, w, part, st.nrm2, counter, st.done);
+        if (e == cudaSuccess) e = krylov_step(L, n, j, m, w, dinv, z, st, p->rtol * bnorm);
       }
-      const double r = std::hypot(h[j], h[j + 1]);
-      cs[j] = r > 0.0 ? h[j] / r : 1.0;
-      sn[j] = r > 0.0 ? h[j + 1] / r : 0.0;
-      h[j] = r;
-      h[j + 1] = 0.0;
-      g[j + 1] = -sn[j] * g[j];
-      g[j] = cs[j] * g[j];
-      for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = h[i];
-      ++total;
-      jdone = j + 1;
-      if (hn > 0.0 && e == cudaSuccess) e = krylov_scaled_copy(L, n, w, 1.0 / hn, w);
-      if (std::fabs(g[j + 1]) <= p->rtol * bnorm || !(hn > 0.0)) break;
+      read(flags, st.jdone, sizeof(flags));
+      if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     }
+    const int jdone = flags[0];
     if (e != cudaSuccess || jdone == 0) break;
+    total += jdone;
+    read(H.data(), st.H, sizeof(double) * (size_t)jdone * (m + 1));
+    read(g.data(), st.g, sizeof(double) * (m + 1));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) break;
     // y = H^-1 g (upper triangular), x += D^-1 V y
     std::vector<double> y(jdone);
     for (int i = jdone - 1; i >= 0; --i) {
       double s = g[i];
-      for (int c = i + 1; c < jdone; ++c) s -= H[(size_t)i * m + c] * y[c];
-      y[i] = H[(size_t)i * m + i] != 0.0 ? s / H[(size_t)i * m + i] : 0.0;
+      for (int c = i + 1; c < jdone; ++c) s -= H[(size_t)c * (m + 1) + i] * y[c];
+      const double d = H[(size_t)i * (m + 1) + i];
+      y[i] = d != 0.0 ? s / d : 0.0;
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hdev, y.data(), sizeof(double) * jdone, cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = krylov_update(L, n, jdone, V, hdev, dinv, x);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ydev, y.data(), sizeof(double) * jdone, cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = krylov_update(L, n, jdone, V, ydev, dinv, x);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // y (host) stays valid until the copy ran
   }
   release();

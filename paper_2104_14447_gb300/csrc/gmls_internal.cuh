@@ -325,13 +325,37 @@ cudaError_t launch_csr_spmv(const Launch& L, int64_t n_rows, const int64_t* row_
                             const double* val, const double* x, double* y, int32_t* long_rows, int32_t* n_long,
                             double* partial);
 
+// the same with the long rows already queued by an earlier call on this matrix
+// (cnt_long of them, known to the host): one launch, y = scale .* (A x) (scale NULL:
+// A x), nothing done where *done is set; counters: int32 [kLongSplitRows], zeroed once
+cudaError_t launch_csr_spmv_queued(const Launch& L, int64_t n_rows, const int64_t* row_ptr, const int32_t* col,
+                                   const double* val, const double* x, double* y, const double* scale,
+                                   const int32_t* long_rows, int cnt_long, double* partial, int32_t* counters,
+                                   const int32_t* done);
+constexpr int kLongSplitRows = 64;  // long rows cut into slices at once
+
 // ------------------------------------------------------------- GMRES pieces
 // (krylov.cu) V holds basis vectors [i][n]; partial has
-// krylov_partial_elems(ncols) doubles; every reduction has a fixed order
+// krylov_partial_elems(ncols) doubles; every reduction has a fixed order;
+// counter: an int32 that is zero before the first launch; done (may be NULL): a
+// launch returns at once where it is set
+struct GmresState {     // device arrays of one solve, restart length m
+  double* H;            // [m][m + 1] rotated Hessenberg columns
+  double *cs, *sn, *g;  // [m], [m], [m + 1]
+  double *h1, *h2;      // [m + 2] coefficients of the two Gram-Schmidt passes
+  double* nrm2;         // |w|^2
+  int32_t *jdone, *done;
+};
 size_t krylov_partial_elems(int max_cols);
 cudaError_t krylov_dots(const Launch& L, int64_t n, int ncols, const double* V, const double* w, double* partial,
-                        double* out);
-cudaError_t krylov_axpy(const Launch& L, int64_t n, int ncols, const double* V, const double* h, double* w);
+                        double* out, int32_t* counter, const int32_t* done);
+cudaError_t krylov_axpy(const Launch& L, int64_t n, int ncols, const double* V, const double* h, double* w,
+                        const int32_t* done);
+cudaError_t krylov_axpy_norm(const Launch& L, int64_t n, int ncols, const double* V, const double* h, double* w,
+                             double* partial, double* out, int32_t* counter, const int32_t* done);
+cudaError_t krylov_step(const Launch& L, int64_t n, int j, int m, double* w, const double* dinv, double* z,
+                        const GmresState& st, double target);
+cudaError_t krylov_start(const Launch& L, const GmresState& st, int m, double beta);
 cudaError_t krylov_update(const Launch& L, int64_t n, int ncols, const double* V, const double* y, const double* dinv,
                           double* x);
 cudaError_t krylov_scale(const Launch& L, int64_t n, const double* dinv, const double* v, double* z);

@@ -168,7 +168,6 @@ __global__ void stokes_rhs_kernel(StokesJob j, const double* __restrict__ f, con
 // queue order, and each path sums in a fixed order: repeated calls give the
 // same bits.
 constexpr int64_t kLongRow = 8192;
-constexpr int kLongSplitRows = 64;
 constexpr int kLongSlices = 128;
 constexpr int kSpmvBlock = 256;
 
@@ -263,6 +262,57 @@ __global__ void __launch_bounds__(kSpmvBlock) csr_spmv_long_kernel(const int64_t
   }
 }
 
+// A x with the long rows known: the first row_blocks blocks take the others,
+// eight lanes a row; then kLongSlices blocks a long row, the last of which adds
+// the row's slices
+__global__ void __launch_bounds__(kSpmvBlock) csr_spmv_queued_kernel(
+    int64_t n_rows, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+    const double* __restrict__ val, const double* __restrict__ x, double* __restrict__ y,
+    const double* __restrict__ scale, int row_blocks, const int32_t* __restrict__ long_rows,
+    double* __restrict__ partial, int32_t* __restrict__ counters, const int32_t* __restrict__ done) {
+  __shared__ double part[kSpmvBlock / 32];
+  __shared__ bool last;
+  if (done && *done) return;
+  if ((int)blockIdx.x >= row_blocks) {
+    const int task = blockIdx.x - row_blocks, i = task / kLongSlices, sl = task % kLongSlices;
+    const int64_t r = long_rows[i];
+    const int64_t a = row_ptr[r], len = row_ptr[r + 1] - a;
+    const double s = block_dot(a + len * sl / kLongSlices, a + len * (sl + 1) / kLongSlices, col, val, x, part);
+    if (threadIdx.x == 0) {
+      partial[task] = s;
+      __threadfence();
+      last = atomicAdd(&counters[i], 1) == kLongSlices - 1;
+      if (last) counters[i] = 0;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    double t = 0.0;
+    for (int b = threadIdx.x; b < kLongSlices; b += 32) t += __ldcg(partial + (int64_t)i * kLongSlices + b);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) y[r] = scale ? scale[r] * t : t;
+    return;
+  }
+  const int sub = threadIdx.x & (kRowLanes - 1);
+  const int64_t stride = (int64_t)row_blocks * blockDim.x / kRowLanes;
+  const int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kRowLanes;
+  const int64_t warp_first = r0 - ((threadIdx.x & 31) / kRowLanes);
+  for (int64_t base = warp_first; base < n_rows; base += stride) {
+    const int64_t r = base + ((threadIdx.x & 31) / kRowLanes);
+    double s = 0.0;
+    bool store = false;
+    if (r < n_rows) {
+      const int64_t a = row_ptr[r], e = row_ptr[r + 1];
+      if (e - a <= kLongRow) {
+        for (int64_t p = a + sub; p < e; p += kRowLanes) s = fma(val[p], x[col[p]], s);
+        store = true;
+      }
+    }
+    for (int o = kRowLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, kRowLanes);
+    if (store && sub == 0) y[r] = scale ? scale[r] * s : s;
+  }
+}
+
 __global__ void csr_spmv_long_finish_kernel(double* __restrict__ y, const int32_t* __restrict__ long_rows,
                                             const int32_t* __restrict__ n_long, const double* __restrict__ partial) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -316,6 +366,18 @@ cudaError_t launch_csr_spmv(const Launch& L, int64_t n_rows, const int64_t* row_
   csr_spmv_long_kernel<<<4 * device_sm_count(), kSpmvBlock, 0, L.stream>>>(row_ptr, col, val, x, y, long_rows, n_long, partial);
   csr_spmv_long_finish_kernel<<<1, 512, 0, L.stream>>>(y, long_rows, n_long, partial);
   *L.counter += 3;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_csr_spmv_queued(const Launch& L, int64_t n_rows, const int64_t* row_ptr, const int32_t* col,
+                                   const double* val, const double* x, double* y, const double* scale,
+                                   const int32_t* long_rows, int cnt_long, double* partial, int32_t* counters,
+                                   const int32_t* done) {
+  if (cnt_long < 0 || cnt_long > kLongSplitRows) return cudaErrorInvalidValue;
+  const unsigned row_blocks = grid_for(n_rows * kRowLanes, kSpmvBlock);
+  csr_spmv_queued_kernel<<<row_blocks + (unsigned)cnt_long * kLongSlices, kSpmvBlock, 0, L.stream>>>(
+      n_rows, row_ptr, col, val, x, y, scale, (int)row_blocks, long_rows, partial, counters, done);
+  *L.counter += 1;
   return cudaGetLastError();
 }
 
