@@ -472,7 +472,8 @@ def variant_name(v):
     if v is None:
         return None
     if v < 0:
-        return {-1: "register", -2: "register 16 lanes", -3: "factored div-free", -4: "register 8 lanes"}.get(v, str(v))
+        return {-1: "register", -2: "register 16 lanes", -3: "factored div-free", -4: "register 8 lanes",
+                -5: "semi-normal equations", -6: "FP64 columns"}.get(v, str(v))
     place = {0: "", 1: ", split tiles", 2: ", global tiles"}.get(v >> 3, "")
     return f"{v & 7} warp(s)/target{place}"
 
@@ -637,7 +638,7 @@ def stokes2d_section(ctx, args, prec_name="fp32_refine"):
           and r["precision"] == prec and not r["bucketed"]]
     chosen = variant_name(min(tl, key=lambda r: r["ms"])["variant"]) if tl else None
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "kernel": f"divergence-free stencil launch, 96 x 20 systems ({chosen or 'heuristic'})",
+                "traffic": None, "kernel": f"divergence-free stencil launch, 96 x 20 systems ({chosen or 'chosen by rule'})",
                 "pipe": pipe, "flops_per_target": f_t, "mean_refine_iters": mean_it_df if prec != gmls.FP64 else 0,
                 "flop_count": "2Mn^2 - 2n^3/3 + L (n^2 + 4Mn) + iters L 4Mn, M = 96, n = 20, L = 2",
                 "peak_source": peak_src, "kernel_ms": k_avg * 1e3}

@@ -382,6 +382,8 @@ gmls_status gmls_launch_count(gmls_ctx* ctx, int64_t* launches);
                                     kernel with 32 / 16 / 8 lanes per target (-4: no
                                     Neumann rows); -3 the factored
                                     divergence-free kernel (div-free basis, FP32 path);
+                                    -5 the semi-normal-equation kernel (FP32 path); -6 the
+                                    FP64 kernel of column-owning lanes (no Neumann rows);
                                     G + 8 * P for the
                                     shared-memory kernel with G = 1, 2 or 4 warps per target
                                     and tile placement P (0: both tiles in shared memory;

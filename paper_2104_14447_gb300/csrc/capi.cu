@@ -103,7 +103,7 @@ struct TuneKey {
 };
 struct TuneRecord {
   TuneKey key;
-  int variant;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored, -5 semi-normal, else warps per target
+  int variant;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored, -5 semi-normal, -6 FP64, else warps per target
   float ms;
 };
 
@@ -332,8 +332,9 @@ static cudaError_t launch_sne(gmls_ctx* ctx, const StencilJob& j, int deg, int k
 // warps per target and its tile placements (generic_candidates); the
 // autotuner times each once on up to 8192 targets and the choice is cached
 // per shape.
-static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls_stencil_params* p, bool refine,
+static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gmls_stencil_params* p, bool refine,
                                   int ld, int nmax, int sms, int32_t* counter) {
+  StencilJob j = j0;
   const int dim = j.dim;
   int mr32 = 0, mr16 = 0, mr8 = 0, mr_pref = 0;
   const bool fast_allowed = refine && (p->weight_power % 2 == 0) && !ctx->force_generic;
@@ -359,7 +360,38 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
   // m = 3, 1,024 targets: 28 against 22 us): there the autotuner times the
   // others, unless this context has taken it for the shape before (a shape then
   // keeps its kernel whatever the number of targets).
+
+  // FP64 kernel of column-owning lanes (variant -6), at any size: 1,024 targets
+  // of the smallest system 36 us and a whole step 116 against 159 us with the
+  // timed best of the shared-memory kernel, 32,761 targets 4.3 against 12.4 ms.
+  // Even weight powers, no Neumann rows, lists of at least the basis size.  The targets it hands off
+  // need a list; in an arena with no room for that beside the shared-memory
+  // kernel's global tiles the latter runs alone.
+  bool ok64 = !refine && p->weight_power % 2 == 0 && !p->neumann && !ctx->force_generic && ctx->force_variant <= 0 &&
+              kmax >= (p->basis == GMLS_BASIS_DIVFREE ? gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree) : nmax) &&
+              f64_path_available(p->basis, dim, p->degree, kmax, j.L);
+  struct HandOff {
+    gmls_ctx* ctx;
+    int32_t* p;
+    ~HandOff() { ctx->arena.release(p); }  // stream ordered, as every scratch
+  } hand{ctx, nullptr};
+  if (ok64) {
+    const int v = heuristic_variant(ld, nmax, false);
+    const size_t tiles = v ? ((global_tile_bytes(ld, nmax, false, v_place(v)) + 255) & ~size_t(255)) * 16 * sms : 0;
+    const size_t list = sizeof(int32_t) * (size_t)(j.n_tgt + 1);
+    ok64 = v && ctx->arena.fits(list + 512 + tiles);
+    if (ok64) {
+      hand.p = arena_alloc<int32_t>(ctx, j.n_tgt + 1);
+      if (!hand.p) return fail(ctx, GMLS_ENOMEM, "gmls_stencils: arena exhausted");
+      j.gen_count = hand.p;
+      j.gen_items = hand.p + 1;
+    }
+  }
   auto launch_fast = [&](const StencilJob& jj, int variant) {
+    if (variant == -6) {
+      cudaError_t e = cudaMemsetAsync(jj.gen_count, 0, sizeof(int32_t), ctx->stream);
+      return e == cudaSuccess ? launch_stencils_f64(ctx->launch(), jj, p->degree, kmax, sms) : e;
+    }
     if (variant == -5) return launch_sne(ctx, jj, p->degree, kmax, false, sms);
     if (variant == -3) {
       DfxShape sh;
@@ -386,12 +418,12 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
                          : launch_stencils_fast(ctx->launch(), jj, mr32, 32, sms);
   };
   const TuneKey key{p->basis, dim, p->degree, p->precision, ld, j.L, p->neumann, 0};
-  int choice = 0;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored div-free, else a vcode
+  int choice = 0;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored div-free, -5 semi-normal, -6 FP64, else a vcode
   auto it = ctx->tune.find(key);
   if (ctx->force_variant != 0) {
     const int v = ctx->force_variant;
     const bool ok = (v == -1 && ok32) || (v == -2 && ok16) || (v == -3 && okdfx) || (v == -4 && ok8) ||
-                    (v == -5 && oksne) ||
+                    (v == -5 && oksne) || (v == -6 && ok64) ||
                     (v > 0 && variant_fits(v, ld, nmax, refine));
     if (!ok) return fail(ctx, GMLS_EINVAL, "gmls_stencils: the forced kernel variant is not available for this shape");
     choice = v;
@@ -400,6 +432,8 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
   } else if (oksne && (j.n_tgt >= 2048 || nmax >= 32)) {
     choice = -5;
     ctx->tune[key] = choice;
+  } else if (ok64) {
+    choice = -6;
   } else if (it != ctx->tune.end()) {
     choice = it->second;
   } else if (ctx->autotune && !capturing(ctx)) {
@@ -485,9 +519,9 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j, const gmls
     jg.n_items = j.gen_count;
     // (with uniform neighbour counts the register kernels hand off only Neumann
     // rows or a tile with fewer rows than basis functions)
-    const int vg = heuristic_variant(ld, nmax, true);
-    if (vg && (p->neumann || ld < nmax || choice == -3 || choice == -5))
-      CK(launch_single(ctx, jg, vg, ld, nmax, true, counter, sms), "gmls_stencils hand-off launch");
+    const int vg = heuristic_variant(ld, nmax, refine);
+    if (vg && (p->neumann || ld < nmax || choice == -3 || choice <= -5))
+      CK(launch_single(ctx, jg, vg, ld, nmax, refine, counter, sms), "gmls_stencils hand-off launch");
   } else
     CK(launch_single(ctx, j, choice, ld, nmax, refine, counter, sms), "gmls_stencils launch");
   return GMLS_OK;
@@ -799,10 +833,10 @@ gmls_status gmls_set_option(gmls_ctx* ctx, int32_t option, int64_t value) {
       return GMLS_OK;
     case GMLS_OPT_AUTOTUNE: ctx->autotune = value != 0; return GMLS_OK;
     case GMLS_OPT_FORCE_VARIANT:
-      if (value != 0 && value != -1 && value != -2 && value != -3 && value != -4 && value != -5 &&
+      if (value != 0 && (value < -6 || value > -1) &&
           !(value > 0 && value < 24 && (v_warps((int)value) == 1 || v_warps((int)value) == 2 ||
                                         v_warps((int)value) == 4)))
-        return fail(ctx, GMLS_EINVAL, "gmls_set_option: variant must be 0, -1 .. -5 or G + 8 * P (G 1, 2, 4; P 0, 1, 2)");
+        return fail(ctx, GMLS_EINVAL, "gmls_set_option: variant must be 0, -1 .. -6 or G + 8 * P (G 1, 2, 4; P 0, 1, 2)");
       ctx->force_variant = (int)value;
       return GMLS_OK;
     case GMLS_OPT_POISON:

@@ -258,6 +258,10 @@ cudaError_t sne_launch_shape(int kind, int dim, int deg, int L, bool neu, int km
                              SneShape* s);
 cudaError_t launch_stencils_sne(const Launch& L, const StencilJob& j, int deg, const SneShape& s, bool neu);
 cudaError_t launch_stencils_dfx(const Launch& L, const StencilJob& j, const DfxShape& s);
+// FP64 kernel of column-owning lanes (stencil_f64.cuh); gen_items / gen_count:
+// the targets it leaves to the shared-memory kernel
+bool f64_path_available(int kind, int dim, int deg, int kmax, int L);
+cudaError_t launch_stencils_f64(const Launch& L, const StencilJob& j, int deg, int kmax, int sms);
 
 // -------------------------------------------------------------------- CSR
 // id order of neighbour lists (see nbr_order_kernel): order[off[t] + r] =

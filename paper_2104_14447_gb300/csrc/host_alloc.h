@@ -47,6 +47,12 @@ class FirstFit {
     }
     return nullptr;
   }
+  // whether a block of this size is free now
+  bool fits(size_t bytes) const {
+    for (const auto& f : free_)
+      if (f.second >= bytes) return true;
+    return false;
+  }
   // releasing NULL or a pointer this allocator did not hand out does nothing
   void release(void* p) {
     if (!p) return;

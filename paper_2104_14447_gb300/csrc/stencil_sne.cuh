@@ -118,6 +118,7 @@ __device__ __forceinline__ ff mul_raw(ff a, ff b) {
   return ff(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
 }
 __device__ __forceinline__ float mul_raw(float a, float b) { return a * b; }
+__device__ __forceinline__ double mul_raw(double a, double b) { return a * b; }
 __device__ __forceinline__ ffp add_c(ffp a, float c) {  // a + c, not normalised
   const f2 cc = dup2(c);
   ffp r;
@@ -131,6 +132,7 @@ __device__ __forceinline__ ff add_c(ff a, float c) {
   return ff(s.h, __fadd_rn(s.l, a.l));
 }
 __device__ __forceinline__ float add_c(float a, float c) { return a + c; }
+__device__ __forceinline__ double add_c(double a, float c) { return a + (double)c; }
 __device__ __forceinline__ ffp quick2(f2 h, f2 l) {  // h + l renormalised, |h| >= |l|
   ffp r;
   r.h = add2(h, l);
@@ -295,6 +297,20 @@ struct SneCoef {
   float a, b, c, d, e, f;
 };
 
+// from the moments 2, 4, 6, 8 averaged over the axes
+template <int HI, bool ST>
+__device__ __forceinline__ void sne_coefficients(const float (&mu)[4], SneCoef& cf) {
+  const float i2 = 1.0f / mu[0], den = mu[1] - mu[0] * mu[0], d4 = mu[2] * mu[0] - mu[1] * mu[1];
+  cf.a = ST ? 0.0f : mu[0];
+  cf.b = HI >= 3 ? mu[1] * i2 : 0.0f;
+  const bool full4 = !ST && den > 1e-4f * mu[1];
+  cf.c = HI >= 4 ? (full4 ? (mu[2] - mu[0] * mu[1]) / den : mu[2] / mu[1]) : 0.0f;
+  cf.d = full4 ? cf.c * mu[0] - mu[1] : 0.0f;
+  const bool full5 = d4 > 1e-4f * mu[1] * mu[1];
+  cf.e = HI >= 5 ? (full5 ? (mu[3] * mu[0] - mu[2] * mu[1]) / d4 : mu[3] / mu[2]) : 0.0f;
+  cf.f = HI >= 5 && full5 ? (cf.e * mu[1] - mu[2]) * i2 : 0.0f;
+}
+
 // q_0 .. q_HI of one axis (q[0] unused)
 template <int HI, typename T>
 __device__ __forceinline__ void sne_axis(T x, const SneCoef& k, T (&q)[HI + 1]) {
@@ -310,6 +326,7 @@ __device__ __forceinline__ void sne_axis(T x, const SneCoef& k, T (&q)[HI + 1]) 
 __device__ __forceinline__ ffp sne_one(ffp) { return ffp{dup2(1.0f), dup2(0.0f)}; }
 __device__ __forceinline__ ff sne_one(ff) { return ff(1.0f, 0.0f); }
 __device__ __forceinline__ float sne_one(float) { return 1.0f; }
+__device__ __forceinline__ double sne_one(double) { return 1.0; }
 
 // column I from the axis values (products that columns share are left to the
 // compiler)
@@ -792,17 +809,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
 #pragma unroll
     for (int e = 0; e < 4; ++e) mu[e] = (e < HI) ? gsum<G>(mu[e]) * (mw / (float)D) : 0.0f;
     SneCoef cf;
-    {
-      const float i2 = 1.0f / mu[0], den = mu[1] - mu[0] * mu[0], d4 = mu[2] * mu[0] - mu[1] * mu[1];
-      cf.a = ST ? 0.0f : mu[0];
-      cf.b = HI >= 3 ? mu[1] * i2 : 0.0f;
-      const bool full4 = !ST && den > 1e-4f * mu[1];
-      cf.c = HI >= 4 ? (full4 ? (mu[2] - mu[0] * mu[1]) / den : mu[2] / mu[1]) : 0.0f;
-      cf.d = full4 ? cf.c * mu[0] - mu[1] : 0.0f;
-      const bool full5 = d4 > 1e-4f * mu[1] * mu[1];
-      cf.e = HI >= 5 ? (full5 ? (mu[3] * mu[0] - mu[2] * mu[1]) / d4 : mu[3] / mu[2]) : 0.0f;
-      cf.f = HI >= 5 && full5 ? (cf.e * mu[1] - mu[2]) * i2 : 0.0f;
-    }
+    sne_coefficients<HI, ST>(mu, cf);
     // q, q', q'' at the target (eta = -centroid), float-float: entry (axis, power, derivative)
     float* LT = base + (DF ? Lay::X : Lay::LT);
     if (lane < D) {
