@@ -52,6 +52,9 @@ __global__ void stokes_rowlen_kernel(StokesJob j) {
   }
 }
 
+// A warp per point.  Bound by HBM (reads the stencils, writes 12 B per nonzero);
+// 512 x 512 points, 1.67 GB: 346 us, 4.8 TB/s (the rows one after another, with
+// plain loads: about 400).
 template <int D>
 __global__ void __launch_bounds__(kStokesWarps * 32) stokes_fill_kernel(StokesJob j) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -63,19 +66,36 @@ __global__ void __launch_bounds__(kStokesWarps * 32) stokes_fill_kernel(StokesJo
     const int kvd = kv * D;
     const double* acc = j.w_cc + ov * D * D;  // this point's curl curl weights
     if (!j.bflag[I]) {
+      // a column and its place in the list serve all D rows; read-only loads, so
+      // that those of several entries are in flight above the stores
+      int64_t rs[D];
 #pragma unroll
-      for (int c = 0; c < D; ++c) {
-        const int64_t r = I * D + c, s = j.row_ptr[r];
-        for (int e = lane; e < kvd; e += 32) {
-          const int q = e / D, cc = e - q * D;
-          const int pv = j.order_v[ov + q];
-          j.col[s + e] = j.idx_v[ov + pv] * D + cc;
-          j.val[s + e] = __dmul_rn(nu, acc[(int64_t)c * kvd + pv * D + cc]);
+      for (int c = 0; c < D; ++c) rs[c] = j.row_ptr[I * D + c];
+#pragma unroll 3
+      for (int e = lane; e < kvd; e += 32) {
+        const int q = e / D, cc = e - q * D;
+        const int pv = __ldg(j.order_v + ov + q);
+        const int32_t cv = __ldg(j.idx_v + ov + pv) * D + cc;
+        double a[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) a[c] = __ldg(acc + (int64_t)c * kvd + pv * D + cc);
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          j.col[rs[c] + e] = cv;
+          j.val[rs[c] + e] = __dmul_rn(nu, a[c]);
         }
-        for (int e = lane; e < kp; e += 32) {
-          const int pp = j.order_p[op + e];
-          j.col[s + kvd + e] = (int32_t)(nd + j.idx_p[op + pp]);
-          j.val[s + kvd + e] = j.w_grad[op * D + (int64_t)c * kp + pp];
+      }
+#pragma unroll 2
+      for (int e = lane; e < kp; e += 32) {
+        const int pp = __ldg(j.order_p + op + e);
+        const int32_t cp = (int32_t)(nd + __ldg(j.idx_p + op + pp));
+        double g[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) g[c] = __ldg(j.w_grad + op * D + (int64_t)c * kp + pp);
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          j.col[rs[c] + kvd + e] = cp;
+          j.val[rs[c] + kvd + e] = g[c];
         }
       }
       // Laplacian row: the staggered stencil on its own list, else the
@@ -87,10 +107,13 @@ __global__ void __launch_bounds__(kStokesWarps * 32) stokes_fill_kernel(StokesJo
       const int16_t* ord = stag ? j.order_s : j.order_p;
       const int32_t* idx = stag ? j.idx_s : j.idx_p;
       const double* wl = stag ? j.w_stag : j.w_lap;
+#pragma unroll 2
       for (int e = lane; e < kl; e += 32) {
-        const int pp = ord[ol + e];
-        j.col[s + e] = (int32_t)(nd + idx[ol + pp]);
-        j.val[s + e] = wl[ol + pp];
+        const int pp = __ldg(ord + ol + e);
+        const int32_t cl = (int32_t)(nd + __ldg(idx + ol + pp));
+        const double v = __ldg(wl + ol + pp);
+        j.col[s + e] = cl;
+        j.val[s + e] = v;
       }
       if (lane == 0) {
         j.col[s + kl] = (int32_t)(nd + n);
@@ -177,6 +200,30 @@ constexpr int kSpmvBlock = 256;
 // 1/64 of the FP32 rate on this GPU.
 constexpr int kRowLanes = 8;
 
+// Bound by the FP64 pipe (84 % busy) and HBM together: 78.8 M entries in 207 us,
+// 4.7 TB/s (with the matrix through L1 and the compiler's own unrolling 270).
+// a lane's entries p, p + 8, .. of its row, in that order; the loads of four
+// entries in flight together, the matrix past L1 (it is read once; x stays)
+__device__ __forceinline__ double row_dot(int64_t p, int64_t e, const int32_t* __restrict__ col,
+                                          const double* __restrict__ val, const double* __restrict__ x) {
+  double s = 0.0;
+  for (; p + 3 * kRowLanes < e; p += 4 * kRowLanes) {
+    double v[4], xv[4];
+    int32_t c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      c[i] = __ldcs(col + p + i * kRowLanes);
+      v[i] = __ldcs(val + p + i * kRowLanes);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) xv[i] = x[c[i]];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s = fma(v[i], xv[i], s);
+  }
+  for (; p < e; p += kRowLanes) s = fma(__ldcs(val + p), x[__ldcs(col + p)], s);
+  return s;
+}
+
 __global__ void csr_spmv_kernel(int64_t n_rows, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                 const double* __restrict__ val, const double* __restrict__ x, double* __restrict__ y,
                                 int32_t* __restrict__ long_rows, int32_t* __restrict__ n_long) {
@@ -195,7 +242,7 @@ __global__ void csr_spmv_kernel(int64_t n_rows, const int64_t* __restrict__ row_
       if (e - a > kLongRow) {
         if (sub == 0) long_rows[atomicAdd(n_long, 1)] = (int32_t)r;
       } else {
-        for (int64_t p = a + sub; p < e; p += kRowLanes) s = fma(val[p], x[col[p]], s);
+        s = row_dot(a + sub, e, col, val, x);
         store = true;
       }
     }
@@ -304,7 +351,7 @@ __global__ void __launch_bounds__(kSpmvBlock) csr_spmv_queued_kernel(
     if (r < n_rows) {
       const int64_t a = row_ptr[r], e = row_ptr[r + 1];
       if (e - a <= kLongRow) {
-        for (int64_t p = a + sub; p < e; p += kRowLanes) s = fma(val[p], x[col[p]], s);
+        s = row_dot(a + sub, e, col, val, x);
         store = true;
       }
     }
