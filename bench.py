@@ -103,10 +103,10 @@ def src_sha(*names):
 # DRAM bytes (read + write) per launch measured by ncu on the timed launch
 # (dram__bytes_read.sum + dram__bytes_write.sum, one pass), with the hash of
 # the kernel sources it was taken on; a different hash reports null
-DFX_TRAFFIC = {"bytes": 700560384 + 10561089536, "sha": "f5e8cff84e6f2b6f",
-               "sources": ("stencil_dfx.cuh", "stencil_fast.cuh", "ff.cuh"),
+SNE_TRAFFIC = {"bytes": 723164416 + 10174838016, "sha": "6fcfdf1d0f63de67",
+               "sources": ("stencil_sne.cuh", "sne_d3.cu", "stencil_fast.cuh", "ff.cuh"),
                "command": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none --nvtx "
-                          "--nvtx-include porous_step/ -k regex:stencil_dfx -c 1 python bench.py --no-secondary "
+                          "--nvtx-include porous_step/ -k regex:stencil_sne -c 3 python bench.py --no-secondary "
                           "--no-e2e --no-cpu-baseline --steps 1 --warmup 3"}
 
 
@@ -320,16 +320,16 @@ def run_headline(args, rank, world, local_rank):
     p32, p64, peak_src = alu_peaks(dev)
     f_t = alg_flops(3 * P_K_DIVFREE, 50, 3, mean_it_df)
     achieved = n * f_t / k_avg / 1e12
-    sha = src_sha(*DFX_TRAFFIC["sources"])
-    traffic = DFX_TRAFFIC["bytes"] if DFX_TRAFFIC["sha"] == sha else None
+    sha = src_sha(*SNE_TRAFFIC["sources"])
+    traffic = SNE_TRAFFIC["bytes"] if SNE_TRAFFIC["sha"] == sha else None
     out_bytes = n * 3 * P_K_DIVFREE * 3 * 8  # FP64 weights written
     roofline = {"bound": "alu", "achieved": achieved, "peak": p32, "unit": "TFLOP/s", "frac": achieved / p32,
                 "traffic": traffic,
                 "traffic_note": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the timed launch "
-                                 f"({DFX_TRAFFIC['command']})") if traffic else
+                                 f"({SNE_TRAFFIC['command']})") if traffic else
                                 "null: no ncu figure for the current kernel sources",
                 "algorithmic_output_bytes": out_bytes,
-                "kernel": "stencil_dfx_kernel<3, 3> (factored div-free QR, FP32 + float-float refinement; "
+                "kernel": "stencil_sne_kernel<1, 3, 3, ..> (corrected semi-normal equations, FP32 R + float-float; "
                           "240 x 50 systems)",
                 "pipe": "fp32", "flops_per_target": f_t, "mean_refine_iters": mean_it_df,
                 "flop_count": "2Mn^2 - 2n^3/3 + L (n^2 + 4Mn) + iters L 4Mn, M = 240, n = 50, L = 3",

@@ -18,7 +18,7 @@ LIB = os.path.join(BUILD, "libgmls.so")
 SOURCES = ["capi.cu", "nbr.cu", "stencil.cu", "stencil_fast.cu", "noalloc.cu", "serve.cu", "stokes.cu", "krylov.cu", "fast_s2a.cu",
            "fast_s2b.cu", "fast_s2c.cu", "fast_s3a.cu", "fast_s3b.cu", "fast_s3c.cu", "fast_d2.cu", "fast_d3.cu", "fast_g2.cu", "fast_g3.cu", "fast_n.cu", "fast_s2d.cu", "dfx.cu",
            "sne.cu", "sne_s2.cu", "sne_s3.cu", "sne_s3b.cu", "sne_n2.cu", "sne_n3.cu", "sne_g.cu", "sne_d2.cu", "sne_d3.cu", "sne_d3b.cu",
-           "f64.cu", "f64_s2.cu", "f64_s3.cu", "f64_d2.cu", "f64_d3.cu", "f64_g.cu"]
+           "f64.cu", "f64_s2.cu", "f64_d2.cu", "f64_d3.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -7,7 +7,7 @@
 
 namespace gmls {
 
-#define GMLS_F64_TABLES(X) X(S2) X(S3) X(D2) X(D3) X(G)
+#define GMLS_F64_TABLES(X) X(S2) X(D2) X(D3)
 #define GMLS_F64_DECL(T)            \
   extern const F64Entry kF64##T[];  \
   extern const int kF64##T##Count;

@@ -3,6 +3,6 @@
 #include "stencil_f64.cuh"
 
 namespace gmls {
-extern const F64Entry kF64D3[] = {GMLS_F64(1, 3, 2, 8, 16), GMLS_F64(1, 3, 3, 8, 12), GMLS_F64(1, 3, 4, 16, 12)};
+extern const F64Entry kF64D3[] = {GMLS_F64(1, 3, 2, 8, 16), GMLS_F64(1, 3, 4, 16, 12)};
 extern const int kF64D3Count = sizeof(kF64D3) / sizeof(kF64D3[0]);
 }  // namespace gmls

@@ -28,7 +28,12 @@
 // divergence-free 2.64 ms, scalar 1.39 ms; the operators from cloud to CSR 12.4 ->
 // 4.3 ms, of 1,024 targets at degree 2 159 -> 116 us; error against 64-bit
 // references unchanged (3.1e-14, 5.9e-16).
-// Not taken: Neumann rows, odd weight powers, lists shorter than the basis,
+// Taken where the error against 64-bit weights is that of a solve with Q within a
+// few percent (measured, new / old): 2D scalar 0.9 to 1.07, 2D divergence-free 0.92
+// to 1.02, 3D divergence-free degree 2 1.03, degree 4 1.04.  Not built: 3D scalar
+// (1.1 to 1.6), 3D divergence-free degree 3 (1.2) and the staggered basis (4 to 8:
+// its columns vanish at the target and have no constant to be orthogonal to).
+// Not taken besides: Neumann rows, odd weight powers, lists shorter than the basis,
 // systems with max / min |r_ii| above 1e5: those targets keep the
 // shared-memory kernel (their status bits come from its factor).
 #pragma once
@@ -204,12 +209,13 @@ template <int KIND, int D, int DEG, int G, int P, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, const F64Tab ftab, int kp) {
   using Dm = SneDims<KIND, D, DEG, false>;
   using Lay = F64Lay<KIND, D, DEG, G, P>;
-  constexpr bool DF = Dm::DF, ST = Dm::ST;
+  constexpr bool DF = Dm::DF;
   constexpr int LO = Dm::LO, HI = Dm::HI, Q = Dm::Q, N = Dm::N, NC = Dm::NC, NTOP = Dm::NTOP, RHS = Lay::RHS;
   constexpr int SA = (Q + G - 1) / G, SN = (N + G - 1) / G;
   constexpr unsigned FULL = 0xffffffffu;
   static_assert(N == gmls_gen::basis_size(KIND, D, DEG), "basis size");
   static_assert(P % 4 == 0, "chunks of four rows");
+  static_assert(KIND != GMLS_BASIS_STAGGERED, "columns orthogonal to a constant");
   extern __shared__ __align__(16) double smd[];
   const SneTab& tab = ftab.t;
   const int lane = threadIdx.x & (G - 1);
@@ -230,18 +236,9 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
     const int64_t t = j.tgt[to], o0 = j.off[to];
     const int k = (int)(j.off[to + 1] - o0);
     const uint8_t st = j.nbr_status ? j.nbr_status[to] : 0;
-    int self = -1;  // staggered: the target's own entry
-    if constexpr (ST) {
-      int f1 = 0x7fffffff;
-      for (int q = lane; q < k; q += G)
-        if (j.idx[o0 + q] == (int32_t)t) f1 = min(f1, q);
-#pragma unroll
-      for (int o = G / 2; o > 0; o >>= 1) f1 = min(f1, __shfl_xor_sync(FULL, f1, o, G));
-      self = f1 == 0x7fffffff ? -1 : f1;
-    }
     const double eps = j.eps[to];
     // what the shared-memory kernel takes
-    bool hand = have && ((st & GMLS_T_TOO_FEW_NEIGHBOURS) || !(eps > 0.0) || k > kp || k < (DF ? Q : N) || (ST && self < 0));
+    bool hand = have && ((st & GMLS_T_TOO_FEW_NEIGHBOURS) || !(eps > 0.0) || k > kp || k < (DF ? Q : N));
     const int ke = have && !hand ? k : 0;
     const int kw = __reduce_max_sync(FULL, ke);  // the longest list in the warp
     if (kw > 0) {
@@ -282,14 +279,14 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
       mw = 1.0f / gsum<G>(mw);
       float sh[D], mu[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int c = 0; c < D; ++c) sh[c] = ST ? 0.0f : gsum<G>(m1[c]) * mw;
+      for (int c = 0; c < D; ++c) sh[c] = gsum<G>(m1[c]) * mw;
 #pragma unroll 2
       for (int q = lane; q < kr; q += G) {  // (the rows this lane wrote)
         const float wt = (float)SW[q] * (float)SW[q];
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-          double x = X[c * kp + q];
-          if constexpr (!ST) X[c * kp + q] = x = x - (double)sh[c];
+          const double x = X[c * kp + q] - (double)sh[c];
+          X[c * kp + q] = x;
           const float s = (float)x * (float)x;
           float p = wt * s;
 #pragma unroll
@@ -303,7 +300,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
 #pragma unroll
       for (int e = 0; e < 4; ++e) mu[e] = e < HI ? gsum<G>(mu[e]) * (mw / (float)D) : 0.0f;
       SneCoef cf;
-      sne_coefficients<HI, ST>(mu, cf);
+      sne_coefficients<HI, false>(mu, cf);
       // q, q', q'' at the target (eta = -centroid): entry (axis, power, derivative)
       __syncwarp();
       if (lane < D) {
@@ -311,7 +308,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
 #pragma unroll
         for (int c = 1; c < D; ++c)
           if (lane == c) s0 = sh[c];
-        const double x = -(double)s0, tt = x * x, a = cf.a, b = cf.b, cc = cf.c, dd = cf.d, ee = cf.e, ff_ = cf.f;
+        const double x = -(double)s0, tt = x * x, a = cf.a, b = cf.b, cc = cf.c, dd = cf.d;
         double* o = LT + lane * 3 * (HI + 1);
         auto put = [&](int p, double v, double d1, double d2) { o[3 * p] = v, o[3 * p + 1] = d1, o[3 * p + 2] = d2; };
         put(0, 1.0, 0.0, 0.0);
@@ -319,7 +316,6 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
         if constexpr (HI >= 2) put(2, tt - a, 2.0 * x, 2.0);
         if constexpr (HI >= 3) put(3, x * (tt - b), 3.0 * tt - b, 6.0 * x);
         if constexpr (HI >= 4) put(4, tt * (tt - cc) + dd, x * (4.0 * tt - 2.0 * cc), 12.0 * tt - 2.0 * cc);
-        if constexpr (HI >= 5) put(5, x * (tt * (tt - ee) + ff_), tt * (5.0 * tt - 3.0 * ee) + ff_, x * (20.0 * tt - 6.0 * ee));
       }
       for (int r = lane; r < L * NC; r += G) {
         const int l = r / NC, cc = r - l * NC;
@@ -519,9 +515,6 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
       // ---- 5. w = W B y
       const bool live = have && !hand;
       if (live) {
-        double others[ST ? Lay::LMAX : 1];
-#pragma unroll
-        for (double& v : others) v = 0.0;
 #pragma unroll 1
         for (int q = lane; q < ke; q += G) {
           double x[D], m[Q];
@@ -542,28 +535,8 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_f64_kernel(StencilJob j, cons
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const SneDst d = dst[2 * r + e];
-              if (d.p && !(ST && q == self)) __stcs(d.p + (int64_t)q * d.stride, d.sgn < 0.0f ? -v : v);
+              if (d.p) __stcs(d.p + (int64_t)q * d.stride, d.sgn < 0.0f ? -v : v);
             }
-            if constexpr (ST) {
-              if (q != self)
-#pragma unroll
-                for (int l = 0; l < Lay::LMAX; ++l)
-                  if (l == r) others[l] += v;
-            }
-          }
-        }
-        if constexpr (ST) {  // the target's own entry: minus the sum of the others
-          const unsigned mask = G == 32 ? FULL : (((1u << (G & 31)) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-#pragma unroll
-          for (int l = 0; l < Lay::LMAX; ++l) {
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) others[l] += __shfl_xor_sync(mask, others[l], o, G);
-            if (lane == 0 && l < L)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const SneDst d = dst[2 * l + e];
-                if (d.p) d.p[(int64_t)self * d.stride] = d.sgn < 0.0f ? others[l] : -others[l];
-              }
           }
         }
         for (int f = 0; f < j.nout; ++f)
