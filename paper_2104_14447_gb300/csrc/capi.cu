@@ -91,12 +91,15 @@ namespace gmls {
 void set_global_error(const std::string& msg) { g_create_error = msg; }
 }  // namespace gmls
 
+// Everything that decides which kernels take a call: a choice cached for one
+// call serves another only where all of it agrees (odd_power: the kernels that
+// form sqrt(W) as a power of (1 - r/eps) take even weight powers only).
 struct TuneKey {
-  int basis, dim, degree, precision, ld, L, neumann, bucketed;
+  int basis, dim, degree, precision, ld, L, neumann, odd_power, bucketed;
   bool operator<(const TuneKey& o) const {
-    const int a[8] = {basis, dim, degree, precision, ld, L, neumann, bucketed};
-    const int b[8] = {o.basis, o.dim, o.degree, o.precision, o.ld, o.L, o.neumann, o.bucketed};
-    for (int i = 0; i < 8; ++i)
+    const int a[9] = {basis, dim, degree, precision, ld, L, neumann, odd_power, bucketed};
+    const int b[9] = {o.basis, o.dim, o.degree, o.precision, o.ld, o.L, o.neumann, o.odd_power, o.bucketed};
+    for (int i = 0; i < 9; ++i)
       if (a[i] != b[i]) return a[i] < b[i];
     return false;
   }
@@ -417,7 +420,7 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
     return variant == -2 ? launch_stencils_fast(ctx->launch(), jj, mr16, 16, sms)
                          : launch_stencils_fast(ctx->launch(), jj, mr32, 32, sms);
   };
-  const TuneKey key{p->basis, dim, p->degree, p->precision, ld, j.L, p->neumann, 0};
+  const TuneKey key{p->basis, dim, p->degree, p->precision, ld, j.L, p->neumann, p->weight_power % 2, 0};
   int choice = 0;  // -1 / -2 / -4 register kernel (32 / 16 / 8 lanes per target), -3 factored div-free, -5 semi-normal, -6 FP64, else a vcode
   auto it = ctx->tune.find(key);
   if (ctx->force_variant != 0) {
@@ -573,7 +576,7 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
       const int bi = (m - 1) * b.n_classes + rc;
       pl.ld[bi] = b.class_rows[rc];
       pl.nmax[bi] = gmls_gen::basis_size(p->basis, dim, m);
-      const TuneKey key{p->basis, dim, m, p->precision, pl.ld[bi], j.L, p->neumann, 1};
+      const TuneKey key{p->basis, dim, m, p->precision, pl.ld[bi], j.L, p->neumann, p->weight_power % 2, 1};
       auto it = ctx->tune.find(key);
       const int v = (it != ctx->tune.end()) ? it->second : heuristic_variant(pl.ld[bi], pl.nmax[bi], refine);
       pl.G[bi] = v_warps(v);
@@ -623,7 +626,7 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
   for (int m = 1; m <= 4 && !need; ++m)
     for (int rc = 0; rc < b.n_classes; ++rc) {
       if (sne[(m - 1) * b.n_classes + rc] || (!p->degree_per_target && m != p->degree)) continue;
-      const TuneKey key{p->basis, dim, m, p->precision, b.class_rows[rc], j.L, p->neumann, 1};
+      const TuneKey key{p->basis, dim, m, p->precision, b.class_rows[rc], j.L, p->neumann, p->weight_power % 2, 1};
       if (!ctx->tune.count(key)) need = true;
     }
   if (need && ctx->autotune && !ctx->force_generic && !capturing(ctx)) {
@@ -653,7 +656,7 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
       for (int rc = 0; rc < b.n_classes; ++rc) {
         const int bi = (m - 1) * b.n_classes + rc;
         if (sne[bi]) continue;
-        const TuneKey key{p->basis, dim, m, p->precision, b.class_rows[rc], j.L, p->neumann, 1};
+        const TuneKey key{p->basis, dim, m, p->precision, b.class_rows[rc], j.L, p->neumann, p->weight_power % 2, 1};
         if (ctx->tune.count(key)) continue;
         if (cnt[bi] == 0) {  // nothing to time: keep the heuristic (later calls skip this pass)
           ctx->tune[key] = heuristic_variant(b.class_rows[rc], gmls_gen::basis_size(p->basis, dim, m), refine);

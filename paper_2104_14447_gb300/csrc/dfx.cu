@@ -76,7 +76,7 @@ size_t dfx_scratch_bytes(int dim, int deg, int64_t n_tgt, int sms) {
 
 cudaError_t launch_stencils_dfx(const Launch& L, const StencilJob& j, const DfxShape& s) {
   const DfxEntry* ent = dfx_entry(j.dim, j.degree);
-  if (!ent || j.L != j.dim || !j.dscratch) return cudaErrorInvalidValue;
+  if (!ent || j.L != j.dim || !j.dscratch || !whole_half_power(j)) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(ent->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
   if (e != cudaSuccess) return e;
   const DfxTab tab = ent->tab();

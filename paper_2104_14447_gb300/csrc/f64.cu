@@ -48,7 +48,7 @@ bool f64_path_available(int kind, int dim, int deg, int kmax, int L) {
 // fewer when there are not enough targets to give every SM such a block.
 cudaError_t launch_stencils_f64(const Launch& L, const StencilJob& j, int deg, int kmax, int sms) {
   const F64Entry* e = f64_entry(j.kind, j.dim, deg, j.L);
-  if (!e || !j.gen_items || !j.gen_count) return cudaErrorInvalidValue;
+  if (!e || !j.gen_items || !j.gen_count || !whole_half_power(j)) return cudaErrorInvalidValue;
   int kp = f64_kp(kmax);
   const size_t wb = warp_bytes(*e, kp);
   int64_t w = (int64_t)std::min<size_t>(kSmemPerBlock / wb, (size_t)e->maxt / 32);

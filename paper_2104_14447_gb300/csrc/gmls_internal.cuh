@@ -181,6 +181,10 @@ struct StencilJob {
   unsigned char* dscratch; // factored div-free kernel: [grid blocks * warps][slot] (DfxShape)
 };
 
+// sqrt(W) = (1 - r / eps)^(p / 2) as a whole power: what every kernel but the
+// shared-memory one forms (its launcher refuses a job of an odd power)
+inline bool whole_half_power(const StencilJob& j) { return j.wpow == 2.0 * j.wpow_half; }
+
 constexpr int kMaxBuckets = 48;
 
 // How one launch of the shared-memory stencil kernel walks its targets.

@@ -72,7 +72,7 @@ size_t sne_scratch_bytes(int kind, int dim, int deg, int L, int kmax, int64_t n_
 
 cudaError_t launch_stencils_sne(const Launch& L, const StencilJob& j, int deg, const SneShape& s, bool neu) {
   const SneEntry* e = sne_entry(j.kind, j.dim, deg, j.L, neu);
-  if (!e || !j.dscratch) return cudaErrorInvalidValue;
+  if (!e || !j.dscratch || !whole_half_power(j)) return cudaErrorInvalidValue;
   cudaError_t r = cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPerBlock);
   if (r != cudaSuccess) return r;
   const SneTab tab = e->tab();

@@ -84,7 +84,7 @@ cudaError_t launch_stencils_fast(const Launch& L, const StencilJob& j, int mr, i
         e.hw == hw)
       ent = &e;
   });
-  if (!ent) return cudaErrorInvalidValue;
+  if (!ent || !whole_half_power(j)) return cudaErrorInvalidValue;
   // warps per block (up to the kernel's limit): the choice with the most
   // resident groups per SM, the largest block among equals
   const int gpw = 32 / hw;  // groups (targets in flight) per warp

@@ -1,0 +1,48 @@
+"""The kernel a stencil call takes: a choice cached for one call must not serve
+another that the kernel does not take (weight powers in turn on one context).
+Bars as for the FP32 + refinement kernels: 1e-9 relative per target and row
+against the FP64 kernel."""
+import pytest
+import torch
+
+from paper_2104_14447_gb300 import gmls, inputs
+from tests.test_gpu_seminormal import _compare
+
+pytestmark = pytest.mark.gpu
+
+G, L, V = gmls.GRAD, gmls.LAPLACIAN, gmls.VEC_LAPLACIAN
+S, F, T = gmls.SCALAR, gmls.DIVFREE, gmls.STAGGERED
+
+
+@pytest.fixture
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2104_14447_gb300 import build
+
+    build.build()
+    c = gmls.Context(0, arena_bytes=2 << 30)
+    c.set_option(gmls.OPT_POISON, 1)  # outputs start as NaN: unwritten entries cannot pass
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("autotune", [1, 0])
+@pytest.mark.parametrize("dim,basis,m,fns,k,axis", [(2, S, 4, [G, L], 36, 72), (2, F, 3, [V], 34, 72), (2, T, 3, [G, L], 36, 72),
+                                                    (3, S, 3, [G, L], 40, 17), (3, F, 3, [V], 80, 13)])
+def test_weight_powers_in_turn(ctx, dim, basis, m, fns, k, axis, autotune):
+    ctx.set_option(gmls.OPT_AUTOTUNE, autotune)
+    x = inputs.jittered_grid(dim, axis, seed=m)
+    nid = ctx.neighbors(ctx.cloud(x), k, 1.5)
+    for power in (4, 3, 1, 4, 5, 2):
+        worst, _ = _compare(ctx, nid, basis, m, fns, k, x.shape[1], forced=False, weight_power=power)
+        assert worst <= 1.0, power
+
+
+@pytest.mark.parametrize("basis,fns", [(S, [G, L]), (F, [V])])
+def test_weight_powers_in_turn_on_uneven_lists(ctx, basis, fns):
+    x = inputs.jittered_grid(2, 72, seed=5)
+    nid = ctx.neighbors(ctx.cloud(x), 24, 1.3, mode=gmls.RADIUS, cap=100)
+    for power in (4, 3, 4):
+        worst, _ = _compare(ctx, nid, basis, 3, fns, 0, x.shape[1], forced=False, weight_power=power)
+        assert worst <= 1.0, power
