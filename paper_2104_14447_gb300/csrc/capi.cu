@@ -361,8 +361,7 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
   // against 0.21 ms scalar, 0.28 against 3.2 ms divergence-free).  Fewer
   // targets of a small system leave most of its groups without work (2D scalar
   // m = 3, 1,024 targets: 28 against 22 us): there the autotuner times the
-  // others, unless this context has taken it for the shape before (a shape then
-  // keeps its kernel whatever the number of targets).
+  // others.
 
   // FP64 kernel of column-owning lanes (variant -6), at any size: 1,024 targets
   // of the smallest system 36 us and a whole step 116 against 159 us with the
@@ -433,8 +432,7 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
   } else if (ctx->force_generic) {
     choice = heuristic_variant(ld, nmax, refine);
   } else if (oksne && (j.n_tgt >= 2048 || nmax >= 32)) {
-    choice = -5;
-    ctx->tune[key] = choice;
+    choice = -5;  // (not cached: the rule costs nothing, and a call's kernel does not depend on earlier calls)
   } else if (ok64) {
     choice = -6;
   } else if (it != ctx->tune.end()) {

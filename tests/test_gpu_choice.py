@@ -46,3 +46,20 @@ def test_weight_powers_in_turn_on_uneven_lists(ctx, basis, fns):
     for power in (4, 3, 4):
         worst, _ = _compare(ctx, nid, basis, 3, fns, 0, x.shape[1], forced=False, weight_power=power)
         assert worst <= 1.0, power
+
+
+@pytest.mark.parametrize("autotune", [1, 0])
+@pytest.mark.parametrize("dim,basis,m,fns,k,axis,large", [(2, S, 3, [G, L], 20, 31, 80), (2, F, 2, [V], 22, 31, 80),
+                                                          (3, S, 2, [G, L], 20, 10, 17)])
+def test_small_cloud_does_not_depend_on_earlier_calls(ctx, dim, basis, m, fns, k, axis, large, autotune):
+    """A large cloud of the same shape on the same context changes nothing."""
+    ctx.set_option(gmls.OPT_AUTOTUNE, autotune)
+    nid = ctx.neighbors(ctx.cloud(inputs.jittered_grid(dim, axis, seed=1)), k, 1.5)
+    nlarge = ctx.neighbors(ctx.cloud(inputs.jittered_grid(dim, large, seed=2)), k, 1.5)
+    out = []
+    for _ in range(2):
+        sid = ctx.stencils(nid, basis, m, fns, precision=gmls.FP32_REFINE)
+        out.append([ctx.weights(sid, fn) for fn in fns])
+        ctx.release(sid)
+        ctx.release(ctx.stencils(nlarge, basis, m, fns, precision=gmls.FP32_REFINE))
+    assert all(torch.equal(a, b) for a, b in zip(*out))
