@@ -53,6 +53,11 @@
 //    enters as its tangential part (the normal part n_c f / |n|^2 goes into beta
 //    alone), so rows along the normal, whose weights nearly vanish, lose nothing
 //    to the difference.
+//  * Range: lambda carries eps^-1 or eps^-2 and the bounds above its squares, which
+//    leave FP32 already at eps = 1e-9 (a cloud of nanometres).  The systems are
+//    solved for lambda 2^(ORDER ee), 2^ee <= eps < 2^(ee + 1), ORDER the highest
+//    power of 1 / eps among the rows: everything is homogeneous in lambda, so no
+//    other bit changes, and sqrt(W) of the last product carries 2^(-ORDER ee).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -197,6 +202,8 @@ __device__ __forceinline__ double sne_to_double(ff a) {
   const double l = __hiloint2double((int)((v & 0x80000000u) | (((v & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(v << 29));
   return h + l;
 }
+// 2^e; zero and infinity beyond the normal range
+__device__ __forceinline__ float sne_exp2(int e) { return __int_as_float(e < -126 ? 0 : (min(e, 128) + 127) << 23); }
 // where the weights of one right-hand side go: entry q at p + q * stride
 struct SneDst {
   double* p;
@@ -706,8 +713,13 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     __syncwarp();
 
     // ---- 1. xi = (x_j - x_T) / eps and sqrt(W) (float-float from the FP64 offsets)
-    const ff inv_eps = recip(ff(j.eps[to]));
+    // 2^ee / eps (of eps / 2^ee), 1 / eps and 1 / eps^2 times 2^(ORDER ee)
+    constexpr int ORDER = !DF && L == D ? 1 : 2;  // (L == D: the gradient alone)
+    auto eps_exponent = [&]() { return min(126, max(-126, ((__double2hiint(j.eps[to]) >> 20) & 0x7ff) - 1023)); };
+    const float pe = sne_exp2(eps_exponent()), pi = sne_exp2(-eps_exponent());
+    const ff inv_eps = recip(ff(j.eps[to] * (double)pi));
     const ff ie2 = inv_eps * inv_eps;
+    [[maybe_unused]] const ff ie1 = ORDER == 1 ? inv_eps : ff(inv_eps.h * pe, inv_eps.l * pe);
     double xt[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) xt[c] = j.x[c * n + t];
@@ -737,7 +749,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
 #pragma unroll
         for (int c = 0; c < D; ++c) {
           const ff d0 = diff_ff(xv[2 * h][c], xt[c]), d1 = diff_ff(xv[2 * h + 1][c], xt[c]);
-          const ffp dx{pk2(d0.h, d1.h), pk2(d0.l, d1.l)};
+          const ffp dx{mul2(pk2(d0.h, d1.h), dup2(pi)), mul2(pk2(d0.l, d1.l), dup2(pi))};
           xi[c] = mul_ff(dx, ie);
           r2 = add_ff(r2, mul_ff(dx, dx));
         }
@@ -984,7 +996,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
           sc *= e < 2 ? 1.0f : e == 2 ? 0.5f : e == 3 ? 1.0f / 6.0f : e == 4 ? 1.0f / 24.0f : 1.0f / 120.0f;
         }
         dmx = fmaxf(dmx, sc);
-        dmn = fminf(dmn, sc);
+        dmn = sc > 0.0f ? fminf(dmn, sc) : 0.0f;  // (zero and NaN)
       }
     }
     dmx = gmax<G>(dmx);
@@ -996,6 +1008,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     // Laplacian (L = 1: the Laplacian alone; Neumann: then the normal derivative);
     // divergence-free: the vector Laplacian
     [[maybe_unused]] ff nv[D], in2;
+    [[maybe_unused]] float fs = 1.0f;  // power of two that brings s_f (about |n| / eps, scaled) to order one
     if constexpr (NEU) {
       ff n2(0.f, 0.f);
 #pragma unroll
@@ -1004,6 +1017,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         n2 = n2 + nv[c] * nv[c];
       }
       in2 = recip(n2);
+      fs = sne_exp2(-eps_exponent() - (((int)((__float_as_uint(n2.h) >> 23) & 0xffu) - 127) >> 1));
     }
     auto lam = [&](int i, ff (&v)[LR]) {
       if constexpr (DF) {
@@ -1029,7 +1043,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         for (int c = 0; c < D; ++c) {
           if (L != D) lap = lap + p[c] * lt(c, i, 2);
           if (L >= D) {
-            v[c < LR ? c : 0] = p[c] * lt(c, i, 1) * inv_eps;
+            v[c < LR ? c : 0] = p[c] * lt(c, i, 1) * ie1;
           }
         }
         if constexpr (NEU) {
@@ -1110,6 +1124,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     bool conv = false, hand = false;
     int used = 0;
     float prev = 0.0f;
+    [[maybe_unused]] bool beta_ok = true;
 #pragma unroll 1
     for (int step = 0; step <= j.max_refine; ++step) {
       const bool pending = active && !ill && !conv && !hand;
@@ -1333,12 +1348,14 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
       float dmax = 0.0f, smax = 0.0f;
       [[maybe_unused]] double others[L];
       [[maybe_unused]] Dot2 pb[LR];
+      [[maybe_unused]] auto scale = [&](ff v) { return ff(v.h * fs, v.l * fs); };
       if constexpr (ST) {
 #pragma unroll
         for (int l = 0; l < L; ++l) others[l] = 0.0;
       }
       // the weights of row q, right-hand side r
       const SneDst* dst = reinterpret_cast<const SneDst*>(base + Lay::DST);
+      const float so = sne_exp2(-ORDER * eps_exponent());
       auto store = [&](int q, int r, ff wv) {
         const double val = sne_to_double(wv);
 #pragma unroll
@@ -1355,7 +1372,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
 #pragma unroll
         for (int d = 0; d < D; ++d) x[d] = XH[d * kp + q];
         sne_columns<D, LO, HI>(x, cf, m);
-        const ffp sw{dup2(SWH[q]), dup2(SWL[q])};
+        const ffp sw{dup2(SWH[q]), dup2(SWL[q])}, swo{dup2(SWH[q] * so), dup2(SWL[q] * so)};
         [[maybe_unused]] ff sf;  // Neumann: the constraint's right-hand side, taken first
         constexpr int PR = (LC + 1) / 2, PF = NEU ? L / 2 : 0;  // pairs; the first one taken
         ulonglong2 sn = S0[PF * kp + q];
@@ -1390,12 +1407,12 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
             smax = fmaxf(smax, fabsf(b1));
           }
           if constexpr (NEU) {
-            if (i == 0) sf = row_of(s1, L & 1);
+            if (i == 0) sf = scale(row_of(s1, L & 1));
 #pragma unroll
             for (int l = 0; l < LR; ++l)
-              if (l >> 1 == pr) pb[l].add_prod(row_of(s1, l & 1), sf);
+              if (l >> 1 == pr) pb[l].add_prod(l == L ? sf : row_of(s1, l & 1), sf);
           } else {
-            const ffp wv = mul_ff(s1, sw);
+            const ffp wv = mul_ff(s1, swo);
             const double v0 = store(q, 2 * pr, row_of(wv, 0));
             double v1 = 0.0;
             if (two) v1 = store(q, 2 * pr + 1, row_of(wv, 1));
@@ -1427,11 +1444,14 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
       }
       if constexpr (NEU) {
         ff bt[L];
+        beta_ok = true;
         const ff ff2 = recip(gsum<G>(pb[L].value()));
 #pragma unroll
         for (int l = 0; l < L; ++l) {
           bt[l] = gsum<G>(pb[l].value()) * ff2;
-          if (pending && lane == 0 && j.beta) j.beta[to * L + l] = to_double(l < D ? bt[l] + nv[l < D ? l : 0] * in2 : bt[l]);
+          beta_ok = beta_ok && fabsf(bt[l].h) < 1e30f;  // (false for NaN)
+          // (s = s_lambda - bt (fs s_f): beta = fs bt)
+          if (pending && lane == 0 && j.beta) j.beta[to * L + l] = to_double(l < D ? scale(bt[l]) + nv[l < D ? l : 0] * in2 : scale(bt[l]));
         }
 #pragma unroll 1
         for (int q = lane; q < ke; q += G) {
@@ -1442,7 +1462,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
             const ulonglong2 v = S0[i * kp + q];
             sp[i] = ffp{v.x, v.y};
           }
-          const ff sf = row_of(sp[L / 2], L & 1), sw(SWH[q], SWL[q]);
+          const ff sf = scale(row_of(sp[L / 2], L & 1)), sw(SWH[q] * so, SWL[q] * so);
 #pragma unroll
           for (int l = 0; l < L; ++l) store(q, l, (row_of(sp[l / 2], l & 1) - bt[l] * sf) * sw);
         }
@@ -1458,6 +1478,8 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         // s0, where no further step reaches them; the shared-memory FP32 kernel,
         // which starts from Q, takes the target
         hand = step == 1 && rho > 5e-5f && j.max_refine > 1;
+        // no finite beta (a zero normal): its weights are that kernel's too
+        if (NEU && !beta_ok) hand = true;
         conv = conv && !hand;
       }
       __syncwarp();
