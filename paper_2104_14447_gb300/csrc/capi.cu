@@ -328,10 +328,47 @@ static cudaError_t launch_sne(gmls_ctx* ctx, const StencilJob& j, int deg, int k
   return e;
 }
 
-// Uniform neighbour counts and degree: one shape.  Candidates: the register
+// From how many targets on a uniform FP32 call takes the semi-normal-equation
+// kernel (reg: a register or factored kernel exists for the shape).  Measured, that
+// kernel against the timed best of the others, microseconds of the whole call:
+//  * bases of 32 functions and more: any size (3D degree-3 divergence-free, 64
+//    targets 134 / 158; 3D degree-4 scalar 108 / 129 and 347 / 745 on 5,000),
+//    but lists above 128 are slower on a handful of targets (scalar degree 4, 252
+//    neighbours: 223 / 156 on one, 273 / 204 on 64, 271 / 891 on 900) and so are
+//    lists near the basis size (38: 500 / 343 on 2,048, 1084 / 1508 on 5,000);
+//  * shapes with only the shared-memory kernel beside it: 2,048 (2D scalar
+//    degree 4, 144 neighbours: 106 / 325);
+//  * lists shorter than 3/2 of the basis: some targets are ill-conditioned enough
+//    to be handed to the shared-memory kernel, a launch of 90 to 230 (2D scalar
+//    degree 4, 18 random neighbours: 281 / 170 on 2,048, 293 / 211 on 5,000,
+//    383 / 387 on 20,000);
+//  * the staggered basis, whose columns have no constant, hands more over: below
+//    twice the basis and at degree 4 from 32,768 (degree 3, 17: 201 / 105 on
+//    5,000, 293 / 234 on 20,000, 622 / 818 on 80,000; degree 4, 48: 320 / 160,
+//    480 / 404, 1204 / 1410), else from 4,096 (3D degree 2, 40: 94 / 74 on
+//    2,048, 117 / 172 on 5,000);
+//  * lists above 400 leave few groups per SM (3D scalar degree 3, 500: 1030 / 913 on
+//    2,500);
+//  * otherwise 3,072 (2D scalar degree 4: 60 / 65 on 2,048, 71 / 108 on 5,000;
+//    3D degree-2 divergence-free, 64: 110 / 97 and 144 / 190).
+static int64_t sne_min_targets(const StencilJob& j, int degree, int kmax, int nmax, bool reg) {
+  const bool scalar = j.kind == GMLS_BASIS_SCALAR, staggered = j.kind == GMLS_BASIS_STAGGERED;
+  const bool tight = 2 * kmax * j.nc < 3 * nmax;
+  if (nmax >= 32) return scalar && tight ? 4096 : scalar && kmax > 128 ? 256 : 0;
+  if (kmax > 400 && j.kind != GMLS_BASIS_DIVFREE) return 8192;
+  if (!reg) return 2048;
+  if (staggered) return kmax < 2 * nmax || degree == 4 ? 32768 : 4096;
+  if (tight && (scalar || j.dim == 2)) return 8192;
+  return 3072;
+}
+
+// Uniform neighbour counts and degree: one shape.  The semi-normal-equation kernel
+// (FP32) and the FP64 kernel of column-owning lanes are chosen by rule; the other
+// candidates are the register
 // kernel with a warp (variant -1), a half warp (variant -2) or 8 lanes
 // (variant -4; not for Neumann rows, which it has no instantiation for) per
-// target, when this shape is instantiated, and the shared-memory kernel with 1, 2 or 4
+// target, when this shape is instantiated, the factored divergence-free kernel
+// (variant -3) and the shared-memory kernel with 1, 2 or 4
 // warps per target and its tile placements (generic_candidates); the
 // autotuner times each once on up to 8192 targets and the choice is cached
 // per shape.
@@ -351,18 +388,9 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
   const bool okdfx = fast_allowed && p->basis == GMLS_BASIS_DIVFREE &&
                      kmax >= gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree) &&
                      dfx_path_available(dim, p->degree, kmax, j.L);
-  // semi-normal-equation kernel (variant -5)
+  // semi-normal-equation kernel (variant -5), from sne_min_targets on
   const bool oksne = fast_allowed && (p->basis != GMLS_BASIS_DIVFREE || kmax >= gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree)) &&
                      sne_path_available(p->basis, dim, p->degree, kmax, j.L, false);
-  // It wins every shape it is built for from about 2,000 targets on (2D scalar
-  // m = 4: 44 against 55 us on 3,969 targets, 0.39 against 0.59 ms on 62,500;
-  // 3D scalar m = 3: 58 / 114 us on 4,096; 3D divergence-free m = 3: 0.29 /
-  // 0.55 ms) and the large systems at any size (3D degree 4, 1,000 targets: 0.11
-  // against 0.21 ms scalar, 0.28 against 3.2 ms divergence-free).  Fewer
-  // targets of a small system leave most of its groups without work (2D scalar
-  // m = 3, 1,024 targets: 28 against 22 us): there the autotuner times the
-  // others.
-
   // FP64 kernel of column-owning lanes (variant -6), at any size: 1,024 targets
   // of the smallest system 36 us and a whole step 116 against 159 us with the
   // timed best of the shared-memory kernel, 32,761 targets 4.3 against 12.4 ms.
@@ -431,7 +459,7 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
     choice = v;
   } else if (ctx->force_generic) {
     choice = heuristic_variant(ld, nmax, refine);
-  } else if (oksne && (j.n_tgt >= 2048 || nmax >= 32)) {
+  } else if (oksne && j.n_tgt >= sne_min_targets(j, p->degree, kmax, nmax, ok32 || ok16 || ok8 || okdfx)) {
     choice = -5;  // (not cached: the rule costs nothing, and a call's kernel does not depend on earlier calls)
   } else if (ok64) {
     choice = -6;

@@ -63,3 +63,32 @@ def test_small_cloud_does_not_depend_on_earlier_calls(ctx, dim, basis, m, fns, k
         ctx.release(sid)
         ctx.release(ctx.stencils(nlarge, basis, m, fns, precision=gmls.FP32_REFINE))
     assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+def _cloud_list(ctx, dim, k, n):
+    axis = int(round(n ** (1.0 / dim)))
+    assert axis ** dim == n
+    return ctx.neighbors(ctx.cloud(inputs.jittered_grid(dim, axis, seed=k)), k, 1.5)
+
+
+def _same_bits(ctx, nid, basis, m, fns, precision, option, value, **kw):
+    """Whether the call's own choice (no timing) gives the bits of the forced kernel."""
+    out = []
+    ctx.set_option(gmls.OPT_AUTOTUNE, 0)
+    for v in (0, value):
+        ctx.set_option(option, v)
+        sid = ctx.stencils(nid, basis, m, fns, precision=precision, **kw)
+        out.append([ctx.weights(sid, fn) for fn in fns])
+        ctx.set_option(option, 0)
+    return all(torch.equal(a.view(torch.int64), b.view(torch.int64)) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("dim,basis,m,fns,k,n,sne", [
+    (2, S, 3, [G, L], 20, 2500, False), (2, S, 3, [G, L], 20, 3600, True), (2, S, 4, [G, L], 18, 3600, False),
+    (2, S, 4, [G, L], 18, 8281, True), (2, S, 4, [G, L], 144, 2116, True), (2, S, 4, [G, L], 144, 1936, False),
+    (2, T, 3, [G, L], 36, 3600, False), (2, T, 3, [G, L], 36, 4900, True), (2, T, 4, [G, L], 48, 4900, False),
+    (3, T, 2, [G, L], 22, 4913, False), (3, F, 3, [V], 80, 343, True), (3, S, 4, [G, L], 84, 125, True),
+    (3, S, 4, [G, L], 140, 216, False), (3, S, 4, [G, L], 38, 2744, False), (2, F, 2, [V], 22, 2500, False)])
+def test_fp32_choice_by_targets_and_list_length(ctx, dim, basis, m, fns, k, n, sne):
+    nid = _cloud_list(ctx, dim, k, n)
+    assert _same_bits(ctx, nid, basis, m, fns, gmls.FP32_REFINE, gmls.OPT_FORCE_VARIANT, -5) == sne
