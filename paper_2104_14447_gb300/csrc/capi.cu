@@ -362,6 +362,39 @@ static int64_t sne_min_targets(const StencilJob& j, int degree, int kmax, int nm
   return 3072;
 }
 
+// Whether a call has the targets for the FP64 kernel of column-owning lanes.
+// Its few lanes a target need a time that grows with the list and hardly with the
+// number of targets until the chip is full; the shared-memory kernel gives a target
+// one to four warps.  Measured (microseconds of the call, this kernel / timed best
+// of the shared-memory kernel):
+//  * 2D scalar degree 2: 12 neighbours 56 / 49 on 384 targets, 55 / 60 on 512; 24:
+//    77 / 62 on 768, 77 / 95 on 1,024; degree 3, 60: 219 / 165 on 1,536, 217 / 229
+//    on 2,048; degree 4, 36: 221 / 225 on 1,024, 222 / 253 on 1,280; 108: 570 / 451 on
+//    2,048, 593 / 846 on 4,096; lists near the basis hand targets off (17: 386 / 344 on
+//    2,048, 388 / 482 on 3,000); beyond 128 the lists leave few groups per SM (200 at
+//    degree 2: 818 / 732 on 8,192);
+//  * 2D divergence-free: degree 2, 22: 97 / 76 on 768, 97 / 120 on 1,024; degree 4,
+//    48: 385 / 316 on 1,024, 387 / 403 on 1,280; 200: 1167 / 1017 on 1,280,
+//    1168 / 1161 on 1,536; 320: 1764 / 1590 on 768, 1766 / 2306 on 1,024;
+//  * 3D divergence-free degree 2, 42: 277 / 230 on 384, 278 / 283 on 512; 200:
+//    690 / 438 on 128, 691 / 858 on 256; degree 4: any size (136: 2550 / 4125 on 32).
+// That holds while the targets fit the chip at once; a second wave doubles this
+// kernel's time, so each wave needs that many (2D divergence-free degree 4, 200, a
+// wave of 2,432: 2311 / 1727 on 2,500, 2309 / 2137 on 3,000, 2311 / 2704 on 4,096).
+static bool f64_enough_targets(const StencilJob& j, int degree, int kmax, int nmax, int sms) {
+  int64_t n = 0;
+  if (j.kind == GMLS_BASIS_SCALAR) {
+    if (kmax > 128) return false;
+    n = degree == 4 && kmax < 2 * nmax ? 2400 : 28 * kmax + 150;
+  } else if (j.dim == 2) {
+    n = kmax > 256 ? 1000 : std::min(8 * kmax + 800, 1650);
+  } else if (degree < 4) {
+    n = 512 - 3 * kmax / 2;
+  }
+  const int64_t wave = f64_wave_targets(j.kind, j.dim, degree, kmax, j.L, sms);
+  return wave > 0 && j.n_tgt >= n * ((j.n_tgt + wave - 1) / wave);
+}
+
 // Uniform neighbour counts and degree: one shape.  The semi-normal-equation kernel
 // (FP32) and the FP64 kernel of column-owning lanes are chosen by rule; the other
 // candidates are the register
@@ -391,13 +424,12 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
   // semi-normal-equation kernel (variant -5), from sne_min_targets on
   const bool oksne = fast_allowed && (p->basis != GMLS_BASIS_DIVFREE || kmax >= gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree)) &&
                      sne_path_available(p->basis, dim, p->degree, kmax, j.L, false);
-  // FP64 kernel of column-owning lanes (variant -6), at any size: 1,024 targets
-  // of the smallest system 36 us and a whole step 116 against 159 us with the
-  // timed best of the shared-memory kernel, 32,761 targets 4.3 against 12.4 ms.
-  // Even weight powers, no Neumann rows, lists of at least the basis size.  The targets it hands off
-  // need a list; in an arena with no room for that beside the shared-memory
-  // kernel's global tiles the latter runs alone.
-  bool ok64 = !refine && p->weight_power % 2 == 0 && !p->neumann && !ctx->force_generic && ctx->force_variant <= 0 &&
+  // FP64 kernel of column-owning lanes (variant -6), where f64_enough_targets: even
+  // weight powers, no Neumann rows, lists of at least the basis size.  The
+  // targets it hands off need a list; in an arena with no room for that beside
+  // the shared-memory kernel's global tiles the latter runs alone.
+  bool ok64 = !refine && p->weight_power % 2 == 0 && !p->neumann && !ctx->force_generic &&
+              (ctx->force_variant == -6 || (ctx->force_variant == 0 && f64_enough_targets(j, p->degree, kmax, nmax, sms))) &&
               kmax >= (p->basis == GMLS_BASIS_DIVFREE ? gmls_gen::basis_size(GMLS_BASIS_SCALAR, dim, p->degree) : nmax) &&
               f64_path_available(p->basis, dim, p->degree, kmax, j.L);
   struct HandOff {

@@ -44,6 +44,14 @@ bool f64_path_available(int kind, int dim, int deg, int kmax, int L) {
   return e && warp_bytes(*e, f64_kp(kmax)) <= kSmemPerBlock;
 }
 
+// targets in flight on the whole chip (0: not available)
+int64_t f64_wave_targets(int kind, int dim, int deg, int kmax, int L, int sms) {
+  const F64Entry* e = f64_entry(kind, dim, deg, L);
+  if (!e) return 0;
+  const size_t w = std::min<size_t>(kSmemPerBlock / warp_bytes(*e, f64_kp(kmax)), (size_t)e->maxt / 32);
+  return (int64_t)w * (32 / e->G) * sms;
+}
+
 // One block per SM of as many warps as its registers and shared memory allow,
 // fewer when there are not enough targets to give every SM such a block.
 cudaError_t launch_stencils_f64(const Launch& L, const StencilJob& j, int deg, int kmax, int sms) {

@@ -265,6 +265,7 @@ cudaError_t launch_stencils_dfx(const Launch& L, const StencilJob& j, const DfxS
 // FP64 kernel of column-owning lanes (stencil_f64.cuh); gen_items / gen_count:
 // the targets it leaves to the shared-memory kernel
 bool f64_path_available(int kind, int dim, int deg, int kmax, int L);
+int64_t f64_wave_targets(int kind, int dim, int deg, int kmax, int L, int sms);
 cudaError_t launch_stencils_f64(const Launch& L, const StencilJob& j, int deg, int kmax, int sms);
 
 // -------------------------------------------------------------------- CSR

@@ -92,3 +92,14 @@ def _same_bits(ctx, nid, basis, m, fns, precision, option, value, **kw):
 def test_fp32_choice_by_targets_and_list_length(ctx, dim, basis, m, fns, k, n, sne):
     nid = _cloud_list(ctx, dim, k, n)
     assert _same_bits(ctx, nid, basis, m, fns, gmls.FP32_REFINE, gmls.OPT_FORCE_VARIANT, -5) == sne
+
+
+@pytest.mark.parametrize("dim,basis,m,fns,k,n,cols", [
+    (2, S, 2, [L, G], 12, 256, False), (2, S, 2, [L, G], 12, 1024, True), (2, S, 2, [L, G], 36, 900, False),
+    (2, S, 4, [G, L], 36, 900, False), (2, S, 4, [G, L], 36, 1296, True), (2, S, 4, [G, L], 17, 2025, False),
+    (2, S, 4, [G, L], 160, 4096, False), (2, F, 3, [V], 34, 900, False), (2, F, 3, [V], 34, 1296, True),
+    (3, F, 2, [V], 42, 343, False), (3, F, 2, [V], 42, 512, True), (3, F, 4, [V], 136, 216, True)])
+def test_fp64_choice_by_targets_and_list_length(ctx, dim, basis, m, fns, k, n, cols):
+    nid = _cloud_list(ctx, dim, k, n)
+    assert _same_bits(ctx, nid, basis, m, fns, gmls.FP64, gmls.OPT_FORCE_VARIANT, -6) == cols
+    assert _same_bits(ctx, nid, basis, m, fns, gmls.FP64, gmls.OPT_FORCE_GENERIC, 1) != cols
