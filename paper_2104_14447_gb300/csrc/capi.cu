@@ -218,7 +218,7 @@ static size_t plan_smem(const BatchPlan& pl, bool fp32) {
 }
 
 // global tile slots for the buckets whose placement needs them:
-// [blocks][groups][slot]
+// [blocks][groups][slot], groups the most of any such bucket
 static bool plan_gscratch(gmls_ctx* ctx, BatchPlan& pl, bool fp32, int grid, void** owned) {
   size_t slot = 0;
   int groups = 1;
@@ -234,6 +234,7 @@ static bool plan_gscratch(gmls_ctx* ctx, BatchPlan& pl, bool fp32, int grid, voi
   pl.gslot_bytes = 0;
   if (!slot) return true;
   pl.gslot_bytes = (slot + 255) & ~size_t(255);
+  pl.gslots = groups;
   *owned = ctx->arena.alloc((size_t)grid * groups * pl.gslot_bytes);
   pl.gscratch = static_cast<unsigned char*>(*owned);
   return *owned != nullptr;

@@ -199,8 +199,10 @@ struct BatchPlan {
   int ld[kMaxBuckets];          // tile rows
   int nmax[kMaxBuckets];        // tile columns
   int gtile[kMaxBuckets];       // tile placement (kPlaceShared / kPlaceSplit / kPlaceGlobal)
-  unsigned char* gscratch;      // [grid blocks][4 / G][gslot_bytes] global tiles
+  unsigned char* gscratch;      // [grid blocks][gslots][gslot_bytes] global tiles
   size_t gslot_bytes;
+  int gslots;                   // slots of a block: the most 4 / G of the buckets, so that
+                                // blocks at work on buckets of different G never share one
 };
 
 struct BucketJob {

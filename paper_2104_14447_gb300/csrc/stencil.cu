@@ -1196,7 +1196,7 @@ __global__ void __launch_bounds__(kBlock, 3) stencil_kernel(StencilJob j, BatchP
       const size_t slice = (REFINE ? make_lay(plan.ld[b], plan.nmax[b], 4, 8, true, place)
                                    : make_lay(plan.ld[b], plan.nmax[b], 8, 8, false, place)).total;
       unsigned char* gslot =
-          place != kPlaceShared ? plan.gscratch + ((size_t)blockIdx.x * gpb + g.gid) * plan.gslot_bytes : nullptr;
+          place != kPlaceShared ? plan.gscratch + ((size_t)blockIdx.x * plan.gslots + g.gid) * plan.gslot_bytes : nullptr;
       process_target<TQ, HP, REFINE>(j, g, smem + (size_t)g.gid * slice, gslot, place, plan.ld[b], plan.nmax[b], to);
     }
   }
