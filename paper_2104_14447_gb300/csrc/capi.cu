@@ -616,11 +616,19 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
   // Buckets of the semi-normal-equation kernel (FP32 path): a launch each, with
   // the shared memory of the bucket's own row class, in place of their tasks of
   // the persistent launch (500,000 mixed-degree targets: 2D 24.8 -> 3.4 ms, 3D
-  // 110 -> 18 ms).
+  // 110 -> 18 ms).  The launches run one after another, so they need enough
+  // targets: the call on a few takes the persistent launch for all buckets
+  // (microseconds with a launch a bucket / with the persistent one, a degree per
+  // target: 2D scalar 277 / 198 on 1,000, 304 / 334 on 4,000; 3D scalar 1163 / 1045
+  // on 4,000, 1215 / 1847 on 8,000; staggered 555 / 519 and 618 / 909;
+  // divergence-free 387 / 304 on 1,000, 418 / 705 on 4,000, 3D 922 / 596 on 300,
+  // 951 / 1575 on 1,000; one degree: 3D scalar degree 3 238 / 109 on 300, 344 / 280
+  // on 1,000, 241 / 481 on 2,000, degree 4 359 / 211 and 334 / 588 on 1,000;
+  // divergence-free 126 / 110 on 500, 279 / 483 on 1,000).
   const bool sne_allowed = refine && (p->weight_power % 2 == 0) && !ctx->force_generic && ctx->force_variant == 0 &&
                            !p->neumann;
   bool sne[kMaxBuckets] = {};
-  bool any_sne = false;
+  int sne_degrees = 0;  // bit m: degree m has such a bucket
   for (int m = 1; m <= 4; ++m)
     for (int rc = 0; rc < b.n_classes; ++rc) {
       const int bi = (m - 1) * b.n_classes + rc;
@@ -628,8 +636,15 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
       const int nq = gmls_gen::basis_size(p->basis == GMLS_BASIS_DIVFREE ? GMLS_BASIS_SCALAR : p->basis, dim, m);
       sne[bi] = sne_allowed && b.class_rows[rc] / j.nc >= nq &&
                 sne_path_available(p->basis, dim, m, b.class_rows[rc] / j.nc, j.L, false);
-      any_sne |= sne[bi];
+      sne_degrees |= (int)sne[bi] << m;
     }
+  const bool several = (sne_degrees & (sne_degrees - 1)) != 0;
+  const bool big = dim == 3 && (p->basis == GMLS_BASIS_STAGGERED || p->degree == 4);
+  const int64_t sne_from = p->basis == GMLS_BASIS_DIVFREE ? (dim == 3 ? 500 : several ? 1700 : 700)
+                           : several                      ? 4500
+                                                          : (big ? 700 : 1250);
+  const bool any_sne = sne_degrees != 0 && j.n_tgt >= sne_from;
+  if (!any_sne) std::fill(std::begin(sne), std::end(sne), false);
   for (int m = 1; m <= 4; ++m)
     for (int rc = 0; rc < b.n_classes; ++rc) {
       const int bi = (m - 1) * b.n_classes + rc;

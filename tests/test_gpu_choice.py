@@ -2,6 +2,9 @@
 another that the kernel does not take (weight powers in turn on one context).
 Bars as for the FP32 + refinement kernels: 1e-9 relative per target and row
 against the FP64 kernel."""
+import math
+
+import numpy as np
 import pytest
 import torch
 
@@ -10,7 +13,7 @@ from tests.test_gpu_seminormal import _compare
 
 pytestmark = pytest.mark.gpu
 
-G, L, V = gmls.GRAD, gmls.LAPLACIAN, gmls.VEC_LAPLACIAN
+G, L, V, C = gmls.GRAD, gmls.LAPLACIAN, gmls.VEC_LAPLACIAN, gmls.CURLCURL
 S, F, T = gmls.SCALAR, gmls.DIVFREE, gmls.STAGGERED
 
 
@@ -65,6 +68,11 @@ def test_small_cloud_does_not_depend_on_earlier_calls(ctx, dim, basis, m, fns, k
     assert all(torch.equal(a, b) for a, b in zip(*out))
 
 
+def _size(dim, basis, degree):
+    full = math.comb(degree + dim, dim)
+    return {S: full, F: dim * full - math.comb(degree - 1 + dim, dim), T: math.comb(degree + 1 + dim, dim) - 1}[basis]
+
+
 def _cloud_list(ctx, dim, k, n):
     axis = int(round(n ** (1.0 / dim)))
     assert axis ** dim == n
@@ -103,3 +111,47 @@ def test_fp64_choice_by_targets_and_list_length(ctx, dim, basis, m, fns, k, n, c
     nid = _cloud_list(ctx, dim, k, n)
     assert _same_bits(ctx, nid, basis, m, fns, gmls.FP64, gmls.OPT_FORCE_VARIANT, -6) == cols
     assert _same_bits(ctx, nid, basis, m, fns, gmls.FP64, gmls.OPT_FORCE_GENERIC, 1) != cols
+
+
+@pytest.mark.parametrize("dim,basis,fns,n,per_target,buckets", [
+    (2, S, [G, L], 900, True, False), (2, S, [G, L], 4900, True, True), (3, S, [G, L], 2197, True, False),
+    (3, S, [G, L], 4913, True, True), (2, S, [G], 900, False, False), (2, S, [G], 1600, False, True),
+    (2, F, [V], 1600, True, False), (2, F, [V], 2025, True, True), (3, F, [V], 343, True, False), (3, F, [V], 729, True, True),
+    (2, T, [G, L], 3600, True, False), (2, T, [G, L], 4900, True, True)])
+def test_uneven_choice_by_targets(ctx, dim, basis, fns, n, per_target, buckets):
+    """One persistent launch for few targets (the bits of the shared-memory
+    kernel), a launch a bucket for many."""
+    axis = int(round(n ** (1.0 / dim)))
+    x = inputs.jittered_grid(dim, axis, seed=4)
+    assert x.shape[1] == n
+    nid = ctx.neighbors(ctx.cloud(x), 24 if dim == 2 else 45, 1.4, mode=gmls.RADIUS, cap=128)
+    kw = dict(degree_per_target=(2 + np.arange(n) % 2).astype(np.int8)) if per_target else {}
+    assert _same_bits(ctx, nid, basis, 0 if per_target else 3, fns, gmls.FP32_REFINE, gmls.OPT_FORCE_GENERIC, 1, **kw) != buckets
+
+
+@pytest.mark.parametrize("dim,basis,fns", [(2, S, [G, L]), (3, S, [G]), (2, F, [V]), (3, F, [C]), (2, T, [G, L])])
+def test_launches_per_bucket_match_fp64(ctx, dim, basis, fns):
+    """Radius lists of every length (some with fewer neighbours than basis
+    functions) and a degree per target, on enough targets for a launch a bucket.
+    Weights of lists of 3/2 of the basis size and more (shorter ones are
+    ill-conditioned: the kernels used before, too, were off by up to 4e-9 there)."""
+    x = inputs.jittered_grid(dim, 70 if dim == 2 else 17, seed=3)
+    n = x.shape[1]
+    deg = (2 + np.arange(n) % (2 if dim == 3 and basis == F else 3)).astype(np.int8)
+    kpt = (6 + (np.arange(n) * 7) % (30 if dim == 2 else 45)).astype(np.int32)
+    nid = ctx.neighbors(ctx.cloud(x), int(kpt.max()), 1.4, mode=gmls.RADIUS, cap=100, k_per_target=kpt)
+    ref = ctx.stencils(nid, basis, 0, fns, precision=gmls.FP64, degree_per_target=deg)
+    sid = ctx.stencils(nid, basis, 0, fns, precision=gmls.FP32_REFINE, degree_per_target=deg)
+    st64, st32 = (ctx.export(h, gmls.X_STATUS, torch.uint8) for h in (ref, sid))
+    bad = gmls.T_RANK_DEFICIENT | gmls.T_UNSUPPORTED | gmls.T_TOO_FEW_NEIGHBOURS
+    assert torch.equal(st64 & bad, st32 & bad)
+    off = ctx.export(nid, gmls.X_NBR_OFFSETS, torch.int64).cpu().numpy()
+    size = {d: _size(dim, basis, d) for d in (2, 3, 4)}
+    long = [t for t in range(n) if 2 * (off[t + 1] - off[t]) * (dim if basis == F else 1) >= 3 * size[int(deg[t])]]
+    assert len(long) > n // 3
+    for fn in fns:
+        _, rows, nc, _ = ctx.stencil_info(sid, fn)
+        a, b = (ctx.weights(h, fn).cpu().numpy() for h in (sid, ref))
+        for t in long:
+            wa, wb = (w[off[t] * rows * nc:off[t + 1] * rows * nc].reshape(rows, -1) for w in (a, b))
+            assert (np.abs(wa - wb).max(1) <= 1e-9 * np.abs(wb).max(1)).all(), t
