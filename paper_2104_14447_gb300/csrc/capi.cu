@@ -284,8 +284,10 @@ static float time_launch(gmls_ctx* ctx, F&& launch) {
   return ms;
 }
 
+// shrink: on an arena that cannot hold the global tiles of a full grid, a smaller
+// one (the blocks take targets from a counter, so any grid is correct)
 static cudaError_t launch_single(gmls_ctx* ctx, const StencilJob& j, int variant, int ld, int nmax, bool fp32,
-                                 int32_t* counter, int sms) {
+                                 int32_t* counter, int sms, bool shrink = false) {
   BatchPlan pl;
   std::memset(&pl, 0, sizeof(pl));
   pl.single = 1;
@@ -298,9 +300,12 @@ static cudaError_t launch_single(gmls_ctx* ctx, const StencilJob& j, int variant
   const size_t smem = plan_smem(pl, fp32);
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int32_t), ctx->stream);
   if (e != cudaSuccess) return e;
-  const int grid = sms * stencil_blocks_per_sm(fp32, smem);
+  int grid = sms * stencil_blocks_per_sm(fp32, smem);
   void* owned = nullptr;
-  if (!plan_gscratch(ctx, pl, fp32, grid, &owned)) return cudaErrorMemoryAllocation;
+  while (!plan_gscratch(ctx, pl, fp32, grid, &owned)) {
+    if (!shrink || grid == 1) return cudaErrorMemoryAllocation;
+    grid = (grid + 1) / 2;
+  }
   Launch L = ctx->launch();
   e = launch_stencils(L, j, pl, fp32, smem, grid);
   ctx->arena.release(owned);  // stream ordered: later work on this stream runs after the kernel
@@ -583,7 +588,7 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
     // rows or a tile with fewer rows than basis functions)
     const int vg = heuristic_variant(ld, nmax, refine);
     if (vg && (p->neumann || ld < nmax || choice == -3 || choice <= -5))
-      CK(launch_single(ctx, jg, vg, ld, nmax, refine, counter, sms), "gmls_stencils hand-off launch");
+      CK(launch_single(ctx, jg, vg, ld, nmax, refine, counter, sms, choice <= -5), "gmls_stencils hand-off launch");
   } else
     CK(launch_single(ctx, j, choice, ld, nmax, refine, counter, sms), "gmls_stencils launch");
   return GMLS_OK;
@@ -790,8 +795,11 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
   if (e == cudaSuccess) e = launch_stencils(L, j, pl, refine, smem, grid);
   ctx->arena.release(owned);
   if (e == cudaSuccess && any_sne) {
+    int ld_sne = 0, nb_sne = 0;  // the largest of its tiles
     for (int bi = 0; bi + 1 < b.nb && e == cudaSuccess; ++bi) {
       if (!sne[bi]) continue;
+      ld_sne = std::max(ld_sne, pl.ld[bi]);
+      nb_sne = std::max(nb_sne, pl.nmax[bi]);
       StencilJob js = j;
       js.degree = bi / b.n_classes + 1;
       js.items = b.items;
@@ -799,13 +807,12 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
       e = launch_sne(ctx, js, js.degree, b.class_rows[bi % b.n_classes] / j.nc, false, sms);
     }
     // its misfits: fewer neighbours than basis functions, staggered lists
-    // without their own target
+    // without their own target, targets of condition above about 300
     StencilJob jg = j;
     jg.items = j.gen_items;
     jg.n_items = j.gen_count;
-    const int nb_max = gmls_gen::basis_size(p->basis, dim, p->degree_per_target ? 4 : p->degree);
-    const int vg = heuristic_variant(ld_max, nb_max, true);
-    if (e == cudaSuccess && vg) e = launch_single(ctx, jg, vg, ld_max, nb_max, true, counter, sms);
+    const int vg = heuristic_variant(ld_sne, nb_sne, true);  // (fits for every row class)
+    if (e == cudaSuccess && vg) e = launch_single(ctx, jg, vg, ld_sne, nb_sne, true, counter, sms, true);
   }
   release();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "gmls_stencils bucketed launch");
