@@ -312,6 +312,15 @@ static cudaError_t launch_single(gmls_ctx* ctx, const StencilJob& j, int variant
   return e;
 }
 
+// Whether the arena holds, beside extra bytes, the semi-normal-equation kernel's
+// slots for a quarter of a full grid.  With less room the kernels that need no slots
+// (or slots of their own) take the call, which then runs where it always did.
+static bool sne_room(gmls_ctx* ctx, const StencilJob& j, int deg, int kmax, bool neu, int sms, size_t extra) {
+  SneShape sh;
+  return sne_launch_shape(j.kind, j.dim, deg, j.L, neu, kmax, j.n_tgt, sms, &sh) == cudaSuccess &&
+         ctx->arena.fits(sh.scratch / 4 + extra);
+}
+
 // The semi-normal-equation kernel on the job's work list; per-group slots for
 // the resident grid, on a small arena a smaller grid (the groups loop over the
 // targets, so any grid is correct).
@@ -497,7 +506,10 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
     choice = v;
   } else if (ctx->force_generic) {
     choice = heuristic_variant(ld, nmax, refine);
-  } else if (oksne && j.n_tgt >= sne_min_targets(j, p->degree, kmax, nmax, ok32 || ok16 || ok8 || okdfx)) {
+  } else if (oksne && j.n_tgt >= sne_min_targets(j, p->degree, kmax, nmax, ok32 || ok16 || ok8 || okdfx) &&
+             sne_room(ctx, j, p->degree, kmax, false, sms, 0) &&
+             (!p->neumann || !sne_path_available(p->basis, dim, p->degree, kmax, j.L, true) ||
+              sne_room(ctx, j, p->degree, kmax, true, sms, 0))) {
     choice = -5;  // (not cached: the rule costs nothing, and a call's kernel does not depend on earlier calls)
   } else if (ok64) {
     choice = -6;
@@ -648,7 +660,10 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
   const int64_t sne_from = p->basis == GMLS_BASIS_DIVFREE ? (dim == 3 ? 500 : several ? 1700 : 700)
                            : several                      ? 4500
                                                           : (big ? 700 : 1250);
-  const bool any_sne = sne_degrees != 0 && j.n_tgt >= sne_from;
+  bool any_sne = sne_degrees != 0 && j.n_tgt >= sne_from;
+  const size_t lists = 8 * (size_t)j.n_tgt + (16u << 10);  // the bucketing's arrays
+  for (int bi = 0; bi + 1 < b.nb && any_sne; ++bi)
+    if (sne[bi]) any_sne = sne_room(ctx, j, bi / b.n_classes + 1, b.class_rows[bi % b.n_classes] / j.nc, false, sms, lists);
   if (!any_sne) std::fill(std::begin(sne), std::end(sne), false);
   for (int m = 1; m <= 4; ++m)
     for (int rc = 0; rc < b.n_classes; ++rc) {

@@ -31,3 +31,30 @@ def test_uneven_batch_does_not_reserve_tiles_for_the_list_capacity():
     total = int(ctx.export(nid, gmls.X_NBR_OFFSETS, torch.int64)[-1])
     assert bool(torch.isfinite(ctx.weights(sid, V)[:total * 9]).all())
     ctx.close()
+
+
+def _lists(ctx, dim, k, n_axis, neu):
+    x = inputs.jittered_grid(dim, n_axis, seed=2)
+    n = x.shape[1]
+    kw = dict(normals=inputs.unit_vectors(5, 6, n, dim), bflags=(inputs.uniform(5, 8, n) < 0.3).astype(np.uint8)) if neu else {}
+    return ctx.neighbors(ctx.cloud(x, **kw), k, 1.5)
+
+
+@pytest.mark.parametrize("dim,basis,m,fns,k,n_axis,variant,neu", [
+    (2, S, 4, [G, L], 36, 64, -2, False), (3, S, 3, [G, L], 40, 16, -1, False), (2, T, 3, [G, L], 36, 72, -1, False),
+    (2, S, 4, [G, L], 36, 64, -2, True)])
+def test_call_fits_where_the_register_kernels_do(dim, basis, m, fns, k, n_axis, variant, neu):
+    """A call runs in an arena with no room for the slots of the
+    semi-normal-equation kernel."""
+    big = gmls.Context(0, arena_bytes=1 << 30)
+    nid = _lists(big, dim, k, n_axis, neu)
+    big.set_option(gmls.OPT_FORCE_VARIANT, variant)
+    big.stencils(nid, basis, m, fns, precision=gmls.FP32_REFINE, neumann=neu)
+    peak = big.arena_usage()[1]
+    small = gmls.Context(0, arena_bytes=peak + 512)  # (the buffer's start is rounded up to 256 bytes)
+    small.set_option(gmls.OPT_AUTOTUNE, 0)
+    nid = _lists(small, dim, k, n_axis, neu)
+    sid = small.stencils(nid, basis, m, fns, precision=gmls.FP32_REFINE, neumann=neu)
+    assert all(bool(torch.isfinite(small.weights(sid, fn)).all()) for fn in fns)
+    for c in (big, small):
+        c.close()
