@@ -58,3 +58,28 @@ def test_call_fits_where_the_register_kernels_do(dim, basis, m, fns, k, n_axis, 
     assert all(bool(torch.isfinite(small.weights(sid, fn)).all()) for fn in fns)
     for c in (big, small):
         c.close()
+
+
+@pytest.mark.parametrize("part", [0.9, 0.5, 0.3, 0.1, 0.02])
+@pytest.mark.parametrize("dim,basis,m,fns,k,n_axis", [(3, F, 3, [V], 80, 14), (2, S, 4, [G, L], 36, 64)])
+def test_grid_shrinks_to_the_slots_the_arena_holds(dim, basis, m, fns, k, n_axis, part):
+    """The forced kernel with a part of a full grid's slots: the same bits."""
+    big = gmls.Context(0, arena_bytes=1 << 30)
+    nid = _lists(big, dim, k, n_axis, False)
+    lists = big.arena_usage()[1]
+    big.set_option(gmls.OPT_FORCE_VARIANT, -5)
+    sid = big.stencils(nid, basis, m, fns, precision=gmls.FP32_REFINE)
+    used, peak, _ = big.arena_usage()
+    slots = peak - used
+    assert slots > 1 << 20 and peak > lists
+    room = used + int(part * slots)
+    assert room >= lists
+    small = gmls.Context(0, arena_bytes=room)
+    nid = _lists(small, dim, k, n_axis, False)
+    small.set_option(gmls.OPT_FORCE_VARIANT, -5)
+    sid2 = small.stencils(nid, basis, m, fns, precision=gmls.FP32_REFINE)
+    assert small.arena_usage()[2] - small.arena_usage()[0] < slots  # a full grid's slots cannot fit
+    for fn in fns:
+        assert torch.equal(big.weights(sid, fn), small.weights(sid2, fn))
+    for c in (big, small):
+        c.close()
