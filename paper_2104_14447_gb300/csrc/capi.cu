@@ -1743,18 +1743,19 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
                 "gmls_gmres: bad argument (restart 1..256, max_iter >= 0, rtol > 0, row_scaling 0 or 1, reserved 0)");
   if (is_host_ptr(row_ptr) || is_host_ptr(col) || is_host_ptr(val) || is_host_ptr(b) || is_host_ptr(x))
     return fail(ctx, GMLS_EINVAL, "gmls_gmres: arrays must be device buffers");
-  if (capturing(ctx)) return fail(ctx, GMLS_EBUSY, "gmls_gmres reads the device every iteration: not during capture");
+  if (capturing(ctx)) return fail(ctx, GMLS_EBUSY, "gmls_gmres reads the device between its iterations: not during capture");
   CK(cudaSetDevice(ctx->device), "gmls_gmres");
   const int m = p->restart;
-  constexpr int kGmresChunk = 8;  // iterations queued before the host looks at done
   double* V = arena_alloc<double>(ctx, (size_t)(m + 1) * n);
   double* z = arena_alloc<double>(ctx, n);
   double* dinv = arena_alloc<double>(ctx, n);
   double* part = arena_alloc<double>(ctx, krylov_partial_elems(m + 2));
-  // H, cs, sn, g, h1, h2, |w|^2 / dot results, y
-  double* hdev = arena_alloc<double>(ctx, (size_t)m * (m + 1) + 2 * m + (m + 1) + 2 * (m + 2) + 2 + m);
+  // H of a chunk with (jdone, done) behind it: one copy to the host; then cs, sn, g,
+  // h1 (then y), h2, |w|^2 / dot results
+  const size_t chunk_elems = (size_t)kGmresChunk * (m + 1) + 1;
+  double* hdev = arena_alloc<double>(ctx, chunk_elems + 2 * m + (m + 1) + 2 * (m + 2) + 2);
   int32_t* long_rows = arena_alloc<int32_t>(ctx, n);
-  int32_t* ints = arena_alloc<int32_t>(ctx, 5 + kLongSplitRows);  // n_long, counter, counter, jdone, done, long rows' counters
+  int32_t* ints = arena_alloc<int32_t>(ctx, 3 + kLongSplitRows);  // n_long, counter, counter, long rows' counters
   double* sp_part = arena_alloc<double>(ctx, csr_spmv_partial_elems());
   const bool rs = p->row_scaling != 0;
   double* rinv = rs ? arena_alloc<double>(ctx, n) : nullptr;
@@ -1770,18 +1771,18 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
     }
   GmresState st;
   st.H = hdev;
-  st.cs = st.H + (size_t)m * (m + 1);
+  st.cs = st.H + chunk_elems;
   st.sn = st.cs + m;
   st.g = st.sn + m;
   st.h1 = st.g + (m + 1);
   st.h2 = st.h1 + (m + 2);
   st.nrm2 = st.h2 + (m + 2);
-  double* ydev = st.nrm2 + 2;
-  st.jdone = ints + 3;
-  st.done = ints + 4;
-  int32_t *n_long = ints, *counter = ints + 1, *long_counters = ints + 5;
+  double* ydev = st.h1;
+  st.jdone = reinterpret_cast<int32_t*>(st.cs - 1);
+  st.done = st.jdone + 1;
+  int32_t *n_long = ints, *counter = ints + 1, *long_counters = ints + 3;
   Launch L = ctx->launch();
-  cudaError_t e = cudaMemsetAsync(ints, 0, sizeof(int32_t) * (5 + kLongSplitRows), ctx->stream);
+  cudaError_t e = cudaMemsetAsync(ints, 0, sizeof(int32_t) * (3 + kLongSplitRows), ctx->stream);
   auto read = [&](void* dst, const void* src, size_t bytes) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, ctx->stream);
   };
@@ -1802,7 +1803,7 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
     dot_host(b, b, &bb);
   }
   const double bnorm = std::sqrt(bb);
-  std::vector<double> H((size_t)(m + 1) * m, 0.0), g(m + 1, 0.0);
+  std::vector<double> H((size_t)(m + 1) * m, 0.0), g(m + 1, 0.0), chunk(chunk_elems, 0.0);
   int total = 0, n_queued = -1;  // long rows (-1: not known yet)
   double rel = 0.0;
   // A in -> out (scaled by rows if asked): the first call queues the long rows
@@ -1833,6 +1834,7 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
     const int steps = std::min(m, p->max_iter - total);
     int32_t flags[2] = {0, 0};  // jdone, done
     for (int j = 0; j < steps && e == cudaSuccess && !flags[1];) {
+      const int j0 = j;
       for (int c = 0; c < kGmresChunk && j < steps; ++c, ++j) {
         double* w = V + (size_t)(j + 1) * n;
         spmv(z, w, rinv, st.done);
@@ -1840,16 +1842,17 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
         if (e == cudaSuccess) e = krylov_dots(L, n, j + 1, V, w, part, st.h1, counter, st.done);
         if (e == cudaSuccess) e = krylov_axpy(L, n, j + 1, V, st.h1, w, st.done);
         if (e == cudaSuccess) e = krylov_dots(L, n, j + 1, V, w, part, st.h2, counter, st.done);
-        if (e == cudaSuccess) e = krylov_axpy_norm(L, n, j + 1, V, st.h2, w, part, st.nrm2, counter, st.done);
+        if (e == cudaSuccess) e = krylov_axpy_norm(L, n, j + 1, V, st.h2, w, sp_part, st.nrm2, counter, st.done);
         if (e == cudaSuccess) e = krylov_step(L, n, j, m, w, dinv, z, st, p->rtol * bnorm);
       }
-      read(flags, st.jdone, sizeof(flags));
+      read(chunk.data(), st.H, sizeof(double) * chunk_elems);
       if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+      std::memcpy(flags, &chunk[chunk_elems - 1], sizeof(flags));
+      std::copy_n(chunk.data(), (size_t)(j - j0) * (m + 1), H.data() + (size_t)j0 * (m + 1));
     }
     const int jdone = flags[0];
     if (e != cudaSuccess || jdone == 0) break;
     total += jdone;
-    read(H.data(), st.H, sizeof(double) * (size_t)jdone * (m + 1));
     read(g.data(), st.g, sizeof(double) * (m + 1));
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) break;

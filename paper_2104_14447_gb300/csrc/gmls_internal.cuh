@@ -346,12 +346,13 @@ cudaError_t launch_csr_spmv_queued(const Launch& L, int64_t n_rows, const int64_
 constexpr int kLongSplitRows = 64;  // long rows cut into slices at once
 
 // ------------------------------------------------------------- GMRES pieces
-// (krylov.cu) V holds basis vectors [i][n]; partial has
-// krylov_partial_elems(ncols) doubles; every reduction has a fixed order;
+// (krylov.cu) V holds basis vectors [i][n]; partial has krylov_partial_elems(ncols)
+// doubles, krylov_axpy_norm's csr_spmv_partial_elems(); every reduction has a fixed order;
 // counter: an int32 that is zero before the first launch; done (may be NULL): a
 // launch returns at once where it is set
+constexpr int kGmresChunk = 8;  // iterations queued before the host reads their columns and looks at done
 struct GmresState {     // device arrays of one solve, restart length m
-  double* H;            // [m][m + 1] rotated Hessenberg columns
+  double* H;            // [kGmresChunk][m + 1] rotated Hessenberg columns, column j at j % kGmresChunk
   double *cs, *sn, *g;  // [m], [m], [m + 1]
   double *h1, *h2;      // [m + 2] coefficients of the two Gram-Schmidt passes
   double* nrm2;         // |w|^2

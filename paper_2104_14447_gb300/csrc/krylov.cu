@@ -32,7 +32,8 @@ constexpr int kDotThreads = 128;   // small blocks: an even share of the FP64 wo
 constexpr int kDotChunk = 8;       // basis vectors per block of the dots
 constexpr int kDotRows = 1024;     // rows per block, up to kDotMaxBlocks row ranges
 constexpr int kAxpyThreads = 128;
-constexpr int kDotMaxBlocks = 304;
+constexpr int kDotMaxBlocks = 272;  // (with these partials and the columns of one chunk a solve needs no more of
+                                    // the arena than it did with 304 partials and one column)
 
 // row ranges of the dots: a function of n alone, so the summation order does not
 // depend on the device
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(256) arnoldi_step_kernel(int64_t n, int j, int
       if (fabs(s * g) <= target || !(hn > 0.0)) *st.done = 1;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) st.H[(int64_t)j * (m + 1) + i] = h[i];
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) st.H[(int64_t)(j % kGmresChunk) * (m + 1) + i] = h[i];
     return;
   }
   // (done may be set by the last block meanwhile: the vector is not used then)
@@ -356,7 +357,7 @@ cudaError_t krylov_dots(const Launch& L, int64_t n, int ncols, const double* V, 
   return cudaGetLastError();
 }
 
-size_t krylov_partial_elems(int max_cols) { return std::max<size_t>((size_t)kDotMaxBlocks * max_cols, kAxpyMaxBlocks); }
+size_t krylov_partial_elems(int max_cols) { return (size_t)kDotMaxBlocks * max_cols; }
 
 cudaError_t krylov_axpy(const Launch& L, int64_t n, int ncols, const double* V, const double* h, double* w,
                         const int32_t* done) {

@@ -83,3 +83,26 @@ def test_grid_shrinks_to_the_slots_the_arena_holds(dim, basis, m, fns, k, n_axis
         assert torch.equal(big.weights(sid, fn), small.weights(sid2, fn))
     for c in (big, small):
         c.close()
+
+
+@pytest.mark.parametrize("row_scaling", [False, True])
+@pytest.mark.parametrize("restart", [1, 2, 7, 30, 100, 256])
+def test_gmres_needs_its_basis_and_a_few_vectors(restart, row_scaling):
+    """The arena of a solve: the basis, up to four vectors and reductions of 304
+    partial sums a column."""
+    n, m = 60000, restart
+
+    def up(count, size):
+        return (count * size + 255) // 256 * 256
+
+    need = (up((m + 1) * n, 8) + (3 if row_scaling else 2) * up(n, 8) + up(n, 4) + up(304 * (m + 2), 8) + up(2 * (m + 2), 8) +
+            up(1, 4) + up(64 * 128, 8))
+    ctx = gmls.Context(0, arena_bytes=need + 512)  # (the buffer's start is rounded up to 256 bytes)
+    i = torch.arange(n, device="cuda")
+    col = torch.stack([(i - 1).clamp(min=0), i, (i + 1).clamp(max=n - 1)], 1).reshape(-1).to(torch.int32)
+    val = torch.tensor([-1.0, 4.0, -1.0], device="cuda", dtype=torch.float64).repeat(n)
+    row = torch.arange(n + 1, device="cuda") * 3
+    x, its, rel = ctx.gmres(row, col, val, torch.ones(n, dtype=torch.float64, device="cuda"), restart=m, max_iter=4 * m + 20,
+                            rtol=1e-9, row_scaling=row_scaling)
+    assert its > 0 and rel < 1e-2 and bool(torch.isfinite(x).all())
+    ctx.close()
