@@ -1814,8 +1814,8 @@ gmls_status gmls_gmres(gmls_ctx* ctx, int64_t n, const int64_t* row_ptr, const i
                                  done);
       return;
     }
-    e = launch_csr_spmv(L, n, row_ptr, col, val, in, out, long_rows, n_long, sp_part);
-    if (scale && e == cudaSuccess) e = krylov_scale_in_place(L, n, scale, out);
+    e = launch_csr_spmv(L, n, row_ptr, col, val, in, out, long_rows, n_long, sp_part, done);
+    if (scale && e == cudaSuccess) e = krylov_scale_in_place(L, n, scale, out, done);
   };
   while (e == cudaSuccess) {
     // r = b - A x into V_0

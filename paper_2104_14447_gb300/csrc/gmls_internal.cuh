@@ -332,9 +332,10 @@ cudaError_t launch_stokes_rhs(const Launch& L, const StokesJob& j, const double*
                               const double* div_f, double* b);
 // scratch: long_rows int32 [n_rows], n_long int32, partial double [csr_spmv_partial_elems()]
 size_t csr_spmv_partial_elems();
+// done (may be NULL): no product where *done is set
 cudaError_t launch_csr_spmv(const Launch& L, int64_t n_rows, const int64_t* row_ptr, const int32_t* col,
                             const double* val, const double* x, double* y, int32_t* long_rows, int32_t* n_long,
-                            double* partial);
+                            double* partial, const int32_t* done = nullptr);
 
 // the same with the long rows already queued by an earlier call on this matrix
 // (cnt_long of them, known to the host): one launch, y = scale .* (A x) (scale NULL:
@@ -356,7 +357,7 @@ struct GmresState {     // device arrays of one solve, restart length m
   double *cs, *sn, *g;  // [m], [m], [m + 1]
   double *h1, *h2;      // [m + 2] coefficients of the two Gram-Schmidt passes
   double* nrm2;         // |w|^2
-  int32_t *jdone, *done;
+  int32_t *jdone, *done;  // iterations of the cycle; 0 until its last one, then their number
 };
 size_t krylov_partial_elems(int max_cols);
 cudaError_t krylov_dots(const Launch& L, int64_t n, int ncols, const double* V, const double* w, double* partial,
@@ -377,7 +378,7 @@ cudaError_t krylov_residual(const Launch& L, int64_t n, const double* b, double*
 // row-scaled matrix (1 where either is absent or zero)
 cudaError_t krylov_row_equilibration(const Launch& L, int64_t n, const int64_t* row_ptr, const int32_t* col,
                                      const double* val, double* rinv, double* dinv);
-cudaError_t krylov_scale_in_place(const Launch& L, int64_t n, const double* d, double* v);
+cudaError_t krylov_scale_in_place(const Launch& L, int64_t n, const double* d, double* v, const int32_t* done = nullptr);
 cudaError_t krylov_inverse_diagonal(const Launch& L, int64_t n, const int64_t* row_ptr, const int32_t* col,
                                     const double* val, double* dinv);
 

@@ -10,8 +10,8 @@
 // the new basis vector with its preconditioned copy; every reduction ends in the
 // block that finishes last, and the Hessenberg column's Givens rotations run
 // beside the normalisation on the device.  The host queues kGmresChunk iterations
-// ahead and reads only whether the solve has converged; iterations queued past
-// that point return at once.  (One column read back per iteration and a
+// ahead and reads their columns and whether the solve has converged; the launches of
+// iterations queued past that point return at once.  (One column read back per iteration and a
 // single-block sum of 304 partials per column took 270 us an iteration on 55,297
 // unknowns, of which the matrix and the basis need about 20.)
 // Every reduction has a fixed order (partial sums over fixed row ranges, then
@@ -169,14 +169,15 @@ __global__ void __launch_bounds__(kAxpyThreads) multi_axpy_kernel(int64_t n, int
 
 // End of iteration j: v_{j+1} = w / |w| in place and z = dinv .* v_{j+1}; the
 // last block applies the earlier rotations to the new Hessenberg column, forms
-// the next one and the residual estimate, and sets done when that is at most
-// target (or w vanished).
+// the next one and the residual estimate, and sets done to j + 1 when that is at
+// most target (or w vanished).  The other blocks see zero or j + 1 there in the
+// iteration that ends the cycle, and leave in those queued after it.
 __global__ void __launch_bounds__(256) arnoldi_step_kernel(int64_t n, int j, int m, double* __restrict__ w,
                                                            const double* __restrict__ dinv, double* __restrict__ z,
                                                            GmresState st, double target) {
   if (blockIdx.x == gridDim.x - 1) {
     __shared__ double h[258], cs[256], sn[256], ch[256], sh[256];
-    if (*st.done) return;
+    if (*st.done) return;  // set by an earlier iteration: this block alone writes it
     for (int i = threadIdx.x; i <= j; i += blockDim.x) {
       h[i] = st.h1[i] + st.h2[i];
       cs[i] = i < j ? st.cs[i] : 0.0;
@@ -206,13 +207,14 @@ __global__ void __launch_bounds__(256) arnoldi_step_kernel(int64_t n, int j, int
       st.g[j + 1] = -s * g;
       st.g[j] = c * g;
       *st.jdone = j + 1;
-      if (fabs(s * g) <= target || !(hn > 0.0)) *st.done = 1;
+      if (fabs(s * g) <= target || !(hn > 0.0)) *st.done = j + 1;
     }
     __syncthreads();
     for (int i = threadIdx.x; i <= j; i += blockDim.x) st.H[(int64_t)(j % kGmresChunk) * (m + 1) + i] = h[i];
     return;
   }
-  // (done may be set by the last block meanwhile: the vector is not used then)
+  const int32_t ended = *static_cast<volatile const int32_t*>(st.done);
+  if (ended != 0 && ended <= j) return;
   const double hn = sqrt(fmax(*st.nrm2, 0.0));
   if (!(hn > 0.0)) return;
   const double inv = 1.0 / hn;
@@ -335,7 +337,9 @@ __global__ void __launch_bounds__(256) row_scales_kernel(int64_t n, const int64_
 }
 
 // v = d .* v
-__global__ void scale_in_place_kernel(int64_t n, const double* __restrict__ d, double* v) {
+__global__ void scale_in_place_kernel(int64_t n, const double* __restrict__ d, double* v,
+                                      const int32_t* __restrict__ done) {
+  if (done && *done) return;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
     v[p] = d[p] * v[p];
 }
@@ -425,8 +429,8 @@ cudaError_t krylov_row_equilibration(const Launch& L, int64_t n, const int64_t* 
   return cudaGetLastError();
 }
 
-cudaError_t krylov_scale_in_place(const Launch& L, int64_t n, const double* d, double* v) {
-  scale_in_place_kernel<<<grid_for(n), 256, 0, L.stream>>>(n, d, v);
+cudaError_t krylov_scale_in_place(const Launch& L, int64_t n, const double* d, double* v, const int32_t* done) {
+  scale_in_place_kernel<<<grid_for(n), 256, 0, L.stream>>>(n, d, v, done);
   *L.counter += 1;
   return cudaGetLastError();
 }

@@ -226,7 +226,9 @@ __device__ __forceinline__ double row_dot(int64_t p, int64_t e, const int32_t* _
 
 __global__ void csr_spmv_kernel(int64_t n_rows, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                 const double* __restrict__ val, const double* __restrict__ x, double* __restrict__ y,
-                                int32_t* __restrict__ long_rows, int32_t* __restrict__ n_long) {
+                                int32_t* __restrict__ long_rows, int32_t* __restrict__ n_long,
+                                const int32_t* __restrict__ done) {
+  if (done && *done) return;  // (no long rows queued: the launches after this one have none)
   const int sub = threadIdx.x & (kRowLanes - 1);
   const int64_t stride = ((int64_t)gridDim.x * blockDim.x) / kRowLanes;
   // every lane of the warp runs the same number of iterations (the shuffles
@@ -404,12 +406,12 @@ size_t csr_spmv_partial_elems() { return (size_t)kLongSplitRows * kLongSlices; }
 
 cudaError_t launch_csr_spmv(const Launch& L, int64_t n_rows, const int64_t* row_ptr, const int32_t* col,
                             const double* val, const double* x, double* y, int32_t* long_rows, int32_t* n_long,
-                            double* partial) {
+                            double* partial, const int32_t* done) {
   if (n_rows <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(n_long, 0, sizeof(int32_t), L.stream);
   if (e != cudaSuccess) return e;
   csr_spmv_kernel<<<grid_for(n_rows * kRowLanes, 256), 256, 0, L.stream>>>(n_rows, row_ptr, col, val, x, y,
-                                                                              long_rows, n_long);
+                                                                              long_rows, n_long, done);
   csr_spmv_long_kernel<<<4 * device_sm_count(), kSpmvBlock, 0, L.stream>>>(row_ptr, col, val, x, y, long_rows, n_long, partial);
   csr_spmv_long_finish_kernel<<<1, 512, 0, L.stream>>>(y, long_rows, n_long, partial);
   *L.counter += 3;
