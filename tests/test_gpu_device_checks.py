@@ -28,3 +28,12 @@ def _run(name, tmp_path):
 
 def test_iterations_queued_past_the_end_write_nothing(tmp_path):
     assert "0 of 6" in _run("krylov_check", tmp_path)
+
+
+def test_fp64_reciprocals(tmp_path):
+    """The approximations are good to 2^-19 (20 mantissa bits read, 20 written), so
+    the third-order steps leave 2^-57; what remains is rounding: half a unit of the
+    last place of the result for the reciprocal, and for the root half of the
+    rounding of x y in the step's residual (half a unit) besides."""
+    root, reciprocal = (float(v) for v in _run("f64_math_check", tmp_path).split())
+    assert root <= 1.5 and reciprocal <= 1.0
