@@ -37,7 +37,6 @@ void set_global_error(const std::string& msg);
 int device_sm_count();
 bool dfx_path_available(int dim, int deg, int kmax, int L);
 size_t dfx_scratch_bytes(int dim, int deg, int64_t n_tgt, int sms);
-size_t sne_scratch_bytes(int kind, int dim, int deg, int L, int kmax, int64_t n_tgt, int sms);
 }
 
 namespace {
@@ -81,14 +80,11 @@ size_t estimate_bytes(const gmls_request& r) {
   const size_t rows = (size_t)k * nc;
   size_t tiles = 0;
   if ((size_t)nb * rows * 12 > 100 * 1024) tiles = (size_t)gmls::device_sm_count() * 4 * ((size_t)nb * rows * 12 + 4096);
-  // slots of the factored divergence-free or the semi-normal-equation kernel
-  // (one of them, during its launch)
-  size_t slots = 0;
+  // per-warp slots of the factored divergence-free kernel (during its launch).  Those
+  // of the semi-normal-equation kernel (4 to 20 MB on a full grid) fit in their
+  // place or in the margin, and it runs on fewer where they do not.
   if (r.basis == GMLS_BASIS_DIVFREE && gmls::dfx_path_available((int)d, r.degree, (int)k, (int)d))
-    slots = gmls::dfx_scratch_bytes((int)d, r.degree, n, gmls::device_sm_count()) + 4096;
-  for (int L = 1; L <= (int)d + 1; ++L)
-    slots = std::max(slots, gmls::sne_scratch_bytes(r.basis, (int)d, r.degree, L, (int)k, n, gmls::device_sm_count()) + 4096);
-  tiles += slots;
+    tiles += gmls::dfx_scratch_bytes((int)d, r.degree, n, gmls::device_sm_count()) + 4096;
   const size_t total = cloud + nbrs + stencils + tiles;
   return total + total / 8 + (16u << 20);
 }

@@ -64,12 +64,6 @@ cudaError_t sne_launch_shape(int kind, int dim, int deg, int L, bool neu, int km
   return cudaSuccess;
 }
 
-// global scratch of a launch over n_tgt targets (0 if the shape is not instantiated)
-size_t sne_scratch_bytes(int kind, int dim, int deg, int L, int kmax, int64_t n_tgt, int sms) {
-  SneShape s;
-  return sne_launch_shape(kind, dim, deg, L, false, kmax, n_tgt, sms, &s) == cudaSuccess ? s.scratch : 0;
-}
-
 cudaError_t launch_stencils_sne(const Launch& L, const StencilJob& j, int deg, const SneShape& s, bool neu) {
   const SneEntry* e = sne_entry(j.kind, j.dim, deg, j.L, neu);
   if (!e || !j.dscratch || !whole_half_power(j)) return cudaErrorInvalidValue;

@@ -106,3 +106,20 @@ def test_gmres_needs_its_basis_and_a_few_vectors(restart, row_scaling):
                             rtol=1e-9, row_scaling=row_scaling)
     assert its > 0 and rel < 1e-2 and bool(torch.isfinite(x).all())
     ctx.close()
+
+
+def test_server_admits_what_its_arena_holds():
+    """31,684 points in 64 MiB: results, lists and cloud take 42 MB, the slots come
+    out of the margin; the same bits as in a context with room to spare."""
+    x = inputs.jittered_grid(2, 178, seed=6)
+    srv = gmls.Server(0, arena_bytes=64 << 20, streams=1, max_inflight=1)
+    t = srv.submit(x, S, 4, 36, [G, L])
+    assert srv.wait(t, 60000)
+    ctx = gmls.Context(0, arena_bytes=1 << 30)
+    ctx.set_option(gmls.OPT_AUTOTUNE, 0)
+    sid = ctx.stencils(ctx.neighbors(ctx.cloud(x), 36, 1.5), S, 4, [G, L], precision=gmls.FP32_REFINE)
+    for fn in (G, L):
+        assert torch.equal(srv.result(t, gmls.X_WEIGHTS, torch.float64, fn), ctx.weights(sid, fn).cpu())
+    srv.release(t)
+    srv.close()
+    ctx.close()
