@@ -312,6 +312,14 @@ static cudaError_t launch_single(gmls_ctx* ctx, const StencilJob& j, int variant
   return e;
 }
 
+// The semi-normal-equation kernel sums in units of 2^-43 of a bound: on
+// divergence-free systems it reaches about 1e-11 whatever the tolerance, where the
+// kernels with compensated products reach 1e-12 (errors at refine_tol 1e-11 / 1e-13:
+// 2D degree 4 1.0e-11 / 9.7e-12 against 2.3e-11 / 7.5e-13, 3D degree 3 1.6e-11 /
+// 7.5e-12 against 5.5e-11 / 1.0e-12).  A call that asks for less keeps those.  (Scalar
+// and staggered systems end above 1e-11 with either kind, with this one lower.)
+static bool sne_reaches(const StencilJob& j) { return j.kind != GMLS_BASIS_DIVFREE || j.tol >= 1e-11; }
+
 // Whether the arena holds, beside extra bytes, the semi-normal-equation kernel's
 // slots for a quarter of a full grid.  With less room the kernels that need no slots
 // (or slots of their own) take the call, which then runs where it always did.
@@ -506,7 +514,7 @@ static gmls_status launch_uniform(gmls_ctx* ctx, const StencilJob& j0, const gml
     choice = v;
   } else if (ctx->force_generic) {
     choice = heuristic_variant(ld, nmax, refine);
-  } else if (oksne && j.n_tgt >= sne_min_targets(j, p->degree, kmax, nmax, ok32 || ok16 || ok8 || okdfx) &&
+  } else if (oksne && sne_reaches(j) && j.n_tgt >= sne_min_targets(j, p->degree, kmax, nmax, ok32 || ok16 || ok8 || okdfx) &&
              sne_room(ctx, j, p->degree, kmax, false, sms, 0) &&
              (!p->neumann || !sne_path_available(p->basis, dim, p->degree, kmax, j.L, true) ||
               sne_room(ctx, j, p->degree, kmax, true, sms, 0))) {
@@ -643,7 +651,7 @@ static gmls_status launch_bucketed(gmls_ctx* ctx, const StencilJob& j, const gml
   // on 1,000, 241 / 481 on 2,000, degree 4 359 / 211 and 334 / 588 on 1,000;
   // divergence-free 126 / 110 on 500, 279 / 483 on 1,000).
   const bool sne_allowed = refine && (p->weight_power % 2 == 0) && !ctx->force_generic && ctx->force_variant == 0 &&
-                           !p->neumann;
+                           !p->neumann && sne_reaches(j);
   bool sne[kMaxBuckets] = {};
   int sne_degrees = 0;  // bit m: degree m has such a bucket
   for (int m = 1; m <= 4; ++m)

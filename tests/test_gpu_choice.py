@@ -155,3 +155,22 @@ def test_launches_per_bucket_match_fp64(ctx, dim, basis, fns):
         for t in long:
             wa, wb = (w[off[t] * rows * nc:off[t + 1] * rows * nc].reshape(rows, -1) for w in (a, b))
             assert (np.abs(wa - wb).max(1) <= 1e-9 * np.abs(wb).max(1)).all(), t
+
+
+@pytest.mark.parametrize("dim,m,k,n", [(2, 4, 48, 4900), (3, 3, 80, 2744), (3, 4, 136, 1000), (2, 3, None, 4900)])
+def test_tight_tolerance_on_divergence_free_systems(ctx, dim, m, k, n):
+    """refine_tol 1e-13 ends at the roundings of the float-float residuals, 2^-48
+    times conditions of up to a thousand: 4e-12."""
+    axis = int(round(n ** (1.0 / dim)))
+    x = inputs.jittered_grid(dim, axis, seed=9)
+    cid = ctx.cloud(x)
+    nid = ctx.neighbors(cid, k, 1.5) if k else ctx.neighbors(cid, 34, 1.4, mode=gmls.RADIUS, cap=100)
+    ref = ctx.stencils(nid, F, m, [V], precision=gmls.FP64)
+    sid = ctx.stencils(nid, F, m, [V], precision=gmls.FP32_REFINE, refine_tol=1e-13)
+    off = ctx.export(nid, gmls.X_NBR_OFFSETS, torch.int64)
+    seg = torch.repeat_interleave(torch.arange(dim * n, device="cuda"), ((off[1:] - off[:-1]) * dim).repeat_interleave(dim))
+    total = seg.shape[0]
+    a, b = (ctx.weights(h, V)[:total] for h in (sid, ref))
+    err, top = (torch.zeros(dim * n, device="cuda", dtype=torch.float64).scatter_reduce_(0, seg, v, "amax")
+                for v in ((a - b).abs(), b.abs()))
+    assert float((err / top).max()) <= 4e-12
