@@ -19,7 +19,11 @@
 //    over the axes): kappa is some ten times below that of the monomials, the
 //    error after one step a hundred times.  In the order of the monomials the
 //    change of basis is triangular, so the scaled diagonal of R is that of the
-//    Taylor basis.
+//    Taylor basis.  Averaging needs axes of like extent: an axis along which the
+//    neighbours spread at most a quarter as far as along the widest is stretched by
+//    a power of two (axis c by 2^s_c; the derivatives at the target and the
+//    component-0 parts below carry the factors).  On a 3D cloud flattened 100 times
+//    the common coefficients alone cost three digits (4.8e-9).
 //  * A group of G lanes (8, 16 or 32) owns a target, 32 / G targets a warp.  For
 //    the QR a lane owns whole columns (column c on lane c % G) and the rows
 //    stream through its registers P at a time, each block eliminated against
@@ -607,11 +611,12 @@ struct SneLay {
   // targets' tables of the divergence-free basis (needed before UH .. only)
   static constexpr int E3 = DF ? X + 6 * D * HI1 : X;
   static constexpr int emax(int a, int b) { return a > b ? a : b; }
-  // eta and sqrt(W): float [2 (D + 1)][kp]; root of sum_q (p_q / |A e_q|)^2: float [kp]
+  // eta and sqrt(W): float [2 (D + 1)][kp]; root of sum_q (p_q / |A e_q|)^2: float [kp];
+  // the axes' s_c, eight bits each: int
   static constexpr int XI = up4(emax(emax(E1, E2), E3));
   // group stride: the 32 / G groups of a warp start G banks apart
   __host__ __device__ static int stride(int kp) {
-    const int need = XI + (2 * (D + 1) + 1) * kp;
+    const int need = XI + (2 * (D + 1) + 1) * kp + 1;
     return G == 32 ? ((need + 3) & ~3) : ((need + 31 - G) / 32 * 32 + G);
   }
 };
@@ -647,6 +652,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
   float* SWH = XL + D * kp;
   float* SWL = SWH + kp;
   float* RN = SWL + kp;
+  int* AX = reinterpret_cast<int*>(RN + kp);
   float* UH = base + Lay::UH;
   float* UL = base + Lay::UL;
   float* MG = base + Lay::MG;
@@ -723,9 +729,9 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     double xt[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) xt[c] = j.x[c * n + t];
-    float mw = 0.0f, m1[D];
+    float mw = 0.0f, m1[D], m2[D];
 #pragma unroll
-    for (int c = 0; c < D; ++c) m1[c] = 0.0f;
+    for (int c = 0; c < D; ++c) m1[c] = m2[c] = 0.0f;
     // (the gathers of four rows in flight together)
 #pragma unroll 1
     for (int q0 = 0; q0 < 2 * pw; q0 += 4 * G) {
@@ -772,7 +778,11 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
           const float wt = sv[e] * sv[e];
           mw += wt;
 #pragma unroll
-          for (int c = 0; c < D; ++c) m1[c] = fmaf(wt, row_of(xi[c], e).h, m1[c]);
+          for (int c = 0; c < D; ++c) {
+            const float x = row_of(xi[c], e).h, wx = wt * x;
+            m1[c] += wx;
+            m2[c] = fmaf(wx, x, m2[c]);
+          }
         }
 #pragma unroll
         for (int c = 0; c < D; ++c) {
@@ -789,6 +799,21 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     float sh[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) sh[c] = ST ? 0.0f : gsum<G>(m1[c]) * mw;
+    // axes to stretch (variances; a flat axis below 2^-40 of the widest is left)
+    int ax = 0;
+    {
+      float vmax = 0.0f;
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        m2[c] = fmaf(-sh[c], sh[c], gsum<G>(m2[c]) * mw);
+        vmax = fmaxf(vmax, m2[c]);
+      }
+#pragma unroll
+      for (int c = 0; c < D; ++c)
+        if (m2[c] * 16.0f <= vmax && m2[c] > vmax * 0x1p-40f)
+          ax |= (int)((__float_as_uint(__fdividef(vmax, m2[c])) >> 23) - 127u) >> 1 << (8 * c);
+    }
+    if (lane == 0) *AX = ax;
     __syncwarp();
     float mu[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // moments 2, 4, 6, 8
 #pragma unroll 1
@@ -803,6 +828,12 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         if constexpr (!ST) {
           x = add_c(x, -sh[c]);
           x = quick2(x.h, x.l);
+        }
+        if (ax != 0) {
+          const f2 f = dup2(sne_exp2((ax >> (8 * c)) & 255));
+          x = ffp{mul2(x.h, f), mul2(x.l, f)};
+        }
+        if (!ST || ax != 0) {
           *reinterpret_cast<f2*>(XH + c * kp + 2 * i) = x.h;
           *reinterpret_cast<f2*>(XL + c * kp + 2 * i) = x.l;
         }
@@ -829,10 +860,12 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
 #pragma unroll
       for (int c = 1; c < D; ++c)
         if (lane == c) s0 = sh[c];
-      const ff x(-s0, 0.0f), tt = x * x;
+      const float f = sne_exp2((ax >> (8 * lane)) & 255), f2nd = f * f;  // of the axis and its derivatives
+      const ff x(-s0 * f, 0.0f), tt = x * x;
       float* o = LT + lane * 6 * (HI + 1);
       auto put = [&](int p, ff v, ff d1, ff d2) {
-        o[6 * p] = v.h, o[6 * p + 1] = v.l, o[6 * p + 2] = d1.h, o[6 * p + 3] = d1.l, o[6 * p + 4] = d2.h, o[6 * p + 5] = d2.l;
+        o[6 * p] = v.h, o[6 * p + 1] = v.l, o[6 * p + 2] = d1.h * f, o[6 * p + 3] = d1.l * f;
+        o[6 * p + 4] = d2.h * f2nd, o[6 * p + 5] = d2.l * f2nd;
       };
       const ff zero(0.f, 0.f), one(1.f, 0.f);
       put(0, one, zero, zero);
@@ -864,11 +897,17 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
       }
       return s;
     };
+    // int d_c: times 2^(s_c - s_0)
+    [[maybe_unused]] const float st1 = sne_exp2(((ax >> 8) & 255) - (ax & 255)), st2 = sne_exp2(((ax >> 16) & 255) - (ax & 255));
+    [[maybe_unused]] auto stretch = [&](int c) { return D == 2 || c == 1 ? st1 : st2; };
     // component-0 part of column i < NTOP over values ff v[.] (float-float): main + further term
     [[maybe_unused]] auto comp0 = [&](int i, const float* vh, const float* vl, int stride) {
       const int src = tab.src[i], xs = tab.xslot[i];
       ff r(0.f, 0.f);
-      if (src >= 0) r = ff(tab.mch[i], tab.mcl[i]) * ff(vh[src * stride], vl[src * stride]);
+      if (src >= 0) {
+        const float f = stretch(1 + i / Q);
+        r = ff(tab.mch[i] * f, tab.mcl[i] * f) * ff(vh[src * stride], vl[src * stride]);
+      }
       if (xs >= 0) {
         const float* xc = base + Lay::XC + 2 * xs;
         const int x = tab.xsrc[xs] * stride;
@@ -893,8 +932,9 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
           v = (gc == 3 ? mul_f(a, 3.f) - b : mul_f(b, 4.f) - mul_f(cc, 2.f)) * recip(ff((float)(g0 + 1), 0.f));
         else
           v = mul_f(g0 == 2 ? b * recip(ff(3.f, 0.f)) - a : mul_f(cc, 0.25f) - mul_f(b, 0.5f), (float)gc);
-        base[Lay::XC + 2 * x] = v.h;
-        base[Lay::XC + 2 * x + 1] = v.l;
+        const float f = stretch(c);
+        base[Lay::XC + 2 * x] = v.h * f;
+        base[Lay::XC + 2 * x + 1] = v.l * f;
       }
       __syncwarp();
     }
@@ -967,7 +1007,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         };
         if (col < NTOP) {
           const int b0 = col / Q * Q, cg = col - b0, xs = tab.xslot[col];
-          if (tab.src[col] >= 0) add_column(tab.src[col], -tab.mch[col]);
+          if (tab.src[col] >= 0) add_column(tab.src[col], -tab.mch[col] * stretch(1 + col / Q));
           if (xs >= 0) add_column(tab.xsrc[xs], -base[Lay::XC + 2 * xs]);
           for (int r = 0; r <= cg; ++r) R[rpk<N>(b0 + r, col)] = RA[rpk<Q>(r, cg)];
         } else if (col < N) {
@@ -980,7 +1020,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
       sne_append<PG, SN, N, G>(a, R, base + Lay::VB, lane, par);
       __syncwarp();
     }
-    // 1 / r_ii and the conditioning of the factor on the Taylor scale (1 / b!)
+    // 1 / r_ii and the conditioning of the factor on the Taylor scale (1 / b!, axes as they are)
     float dmx = 0.0f, dmn = 3.0e38f;
 #pragma unroll
     for (int s = 0; s < SN; ++s) {
@@ -994,6 +1034,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         for (int c = 0; c < D; ++c) {
           const int e = tab.e[c][col];
           sc *= e < 2 ? 1.0f : e == 2 ? 0.5f : e == 3 ? 1.0f / 6.0f : e == 4 ? 1.0f / 24.0f : 1.0f / 120.0f;
+          if (ax != 0) sc *= sne_exp2(-e * ((ax >> (8 * c)) & 255));
         }
         dmx = fmaxf(dmx, sc);
         dmn = sc > 0.0f ? fminf(dmn, sc) : 0.0f;  // (zero and NaN)
@@ -1002,6 +1043,23 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     dmx = gmax<G>(dmx);
     dmn = -gmax<G>(-dmn);
     const bool ill = !(dmn * 1.0e6f >= dmx) || !(dmn > 0.0f);
+    // no estimate from one step (which left up to 1e-8) where the columns are far from
+    // orthogonal -- some r_ii below 1/20 of its column, on flattened and rotated
+    // clouds; 99 % of the targets of jittered ones stay above 1/8 -- or few
+    // neighbours carry the weight (powers from 10 on)
+    bool second = j.wpow_half >= 5;
+    [[maybe_unused]] bool skewed = false;
+    if constexpr (!DF) {
+      float off = 0.0f;
+#pragma unroll
+      for (int s = 0; s < SA; ++s)
+        if (s * G + lane < Q) off = fmaxf(off, cn[s] * fabsf(ID[s * G + lane]));
+      off = gmax<G>(off);
+      second |= off > 20.0f;
+      // (the staggered columns then carry roundings of their own, 3e-9 after two steps)
+      skewed = ST && off > 40.0f;
+    }
+    second = second && j.max_refine > 1;
     __syncwarp();
 
     // functional rows at unknown i (float-float): rows of the gradient, then the
@@ -1087,7 +1145,10 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
 #pragma unroll
         for (int c2 = 1; c2 < D; ++c2) {
           const int i = tab.inv[c2][g];
-          if (i >= 0) uv = uv - mul_f(ff(tab.mch[i], tab.mcl[i]), y[i]);
+          if (i >= 0) {
+            const float f = stretch(c2);
+            uv = uv - mul_f(ff(tab.mch[i] * f, tab.mcl[i] * f), y[i]);
+          }
         }
         if constexpr (Lay::Y_IN_U) {
 #pragma unroll 1
@@ -1471,7 +1532,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         // error left ~ |ds| times the contraction, estimated by the correction's
         // relative size (first step) or the ratio of successive corrections
         const float rho = step == 1 ? dmax / fmaxf(smax, 1e-37f) : dmax / fmaxf(prev, 1e-37f);
-        conv = kSafe * dmax * fminf(1.0f, rho) <= tolf * smax;
+        conv = kSafe * dmax * fminf(1.0f, rho) <= tolf * smax && (step > 1 || !second);
         prev = dmax;
         used = step;
         // kappa above about 300: u's cancelling entries leave their roundings in
@@ -1480,6 +1541,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
         hand = step == 1 && rho > 5e-5f && j.max_refine > 1;
         // no finite beta (a zero normal): its weights are that kernel's too
         if (NEU && !beta_ok) hand = true;
+        if (ST && skewed && j.max_refine > 1) hand = true;
         conv = conv && !hand;
       }
       __syncwarp();
