@@ -405,6 +405,9 @@ static int64_t sne_min_targets(const StencilJob& j, int degree, int kmax, int nm
 // kernel's time, so each wave needs that many (2D divergence-free degree 4, 200, a
 // wave of 2,432: 2311 / 1727 on 2,500, 2309 / 2137 on 3,000, 2311 / 2704 on 4,096).
 static bool f64_enough_targets(const StencilJob& j, int degree, int kmax, int nmax, int sms) {
+  // powers from 10 on leave columns far from orthogonal, where a solve without Q
+  // loses digits (2D degree 2, power 20: 2e-11 from the solve with Q, 4.5e-15 at 4)
+  if (j.wpow_half >= 5) return false;
   int64_t n = 0;
   if (j.kind == GMLS_BASIS_SCALAR) {
     if (kmax > 128) return false;

@@ -174,3 +174,10 @@ def test_tight_tolerance_on_divergence_free_systems(ctx, dim, m, k, n):
     err, top = (torch.zeros(dim * n, device="cuda", dtype=torch.float64).scatter_reduce_(0, seg, v, "amax")
                 for v in ((a - b).abs(), b.abs()))
     assert float((err / top).max()) <= 4e-12
+
+
+@pytest.mark.parametrize("power,cols", [(4, True), (8, True), (10, False), (20, False)])
+def test_fp64_choice_by_weight_power(ctx, power, cols):
+    nid = _cloud_list(ctx, 2, 12, 1600)
+    assert _same_bits(ctx, nid, S, 2, [L, G], gmls.FP64, gmls.OPT_FORCE_VARIANT, -6, weight_power=power) == cols
+    assert _same_bits(ctx, nid, S, 2, [L, G], gmls.FP64, gmls.OPT_FORCE_GENERIC, 1, weight_power=power) != cols
