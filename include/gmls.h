@@ -204,7 +204,9 @@ gmls_status gmls_neighbors_prefix(gmls_ctx* ctx, int64_t nbrs_id, int32_t k, dou
  * order.  Weight w satisfies, for every polynomial field q of the basis span,
  * sum w q(x_j) = (L q)(x_T) (plus beta * h for Neumann targets).
  * Besides the weights, a launch takes temporary scratch from the arena for
- * the duration of the kernel: the factored divergence-free kernel about
+ * the duration of the kernel: the semi-normal-equation kernel 4 to 20 MB on a
+ * full grid (with room for less than a quarter of that another kernel takes the
+ * call), the factored divergence-free kernel about
  * 29 KB per resident warp (3D degree 3: 152 SMs x 12 warps, 53 MB; on a
  * smaller arena it runs a smaller grid, down to one block of 12 warps), the
  * shared-memory kernel its global tiles for shapes too large for shared
@@ -369,8 +371,11 @@ gmls_status gmls_launch_count(gmls_ctx* ctx, int64_t* launches);
 /* options of gmls_set_option */
 #define GMLS_OPT_FORCE_GENERIC 0 /* 1: every shape uses the shared-memory tile kernel, not the
                                     warp-per-target register kernel (testing and tuning)    */
-#define GMLS_OPT_AUTOTUNE 1      /* 1 (default): the first gmls_stencils call for a shape times
-                                    the kernel variants (register kernel with a warp or a half
+#define GMLS_OPT_AUTOTUNE 1      /* 1 (default): the semi-normal-equation kernel (FP32) and the
+                                    FP64 kernel of column-owning lanes are chosen by rules on
+                                    shape, targets and list length; where they are not taken,
+                                    the first gmls_stencils call for a shape (and parity of the
+                                    weight power) times the other variants (register kernel with a warp or a half
                                     warp per target; for the divergence-free basis the
                                     factored kernel; 1, 2 or 4 warps per target, and for tiles
                                     that leave one block per SM the split and global tile

@@ -15,6 +15,8 @@ namespace gmls {
 // no spills; 0.165 vs 0.204 ms at 12 warps on 8,192 targets); 3D m = 2 and
 // m = 3 at 12 (3D m = 2 at 24 warps ran at less than half the speed);
 // 2D m = 2, 3 at 24 (the register kernel takes those shapes).
+// Taken below the number of targets from which the semi-normal-equation kernel is,
+// at tolerances that one does not reach, and on arenas without room for its slots.
 static const DfxEntry kDfx[] = {GMLS_DFX(2, 2, 1, 32, 768), GMLS_DFX(2, 3, 2, 64, 768), GMLS_DFX(2, 4, 2, 64, 640),
                                 GMLS_DFX(3, 2, 2, 64, 384), GMLS_DFX(3, 3, 3, 80, 384)};
 

@@ -28,6 +28,8 @@
 // divergence-free 2.64 ms, scalar 1.39 ms; the operators from cloud to CSR 12.4 ->
 // 4.3 ms, of 1,024 targets at degree 2 159 -> 116 us; error against 64-bit
 // references unchanged (3.1e-14, 5.9e-16).
+// G and P as in stencil_sne.cuh, in FP64: P is what 255 registers hold beside the
+// column slots.
 // Taken where the error against 64-bit weights is that of a solve with Q within a
 // few percent (measured, new / old): 2D scalar 0.9 to 1.07, 2D divergence-free 0.92
 // to 1.02, 3D divergence-free degree 2 1.03, degree 4 1.04.  Not built: 3D scalar

@@ -623,7 +623,7 @@ struct SneLay {
 
 // MAXT bounds the registers (65536 / MAXT a thread): the launcher fills an SM
 // with one block of up to MAXT threads.  LS: right-hand sides per product pass
-// (their 4 Q LS accumulators live in registers).
+// (their 2 Q LS accumulators, high and low parts, live in registers).
 template <int KIND, int D, int DEG, int L, int G, int P, int LS, bool NEU, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, const SneTab tab, int kp) {
   using Dm = SneDims<KIND, D, DEG, NEU>;
@@ -1580,6 +1580,19 @@ struct SneEntry {
   SneTab (*tab)();
 };
 
+// What the tables' G, P, LS and MAXT follow:
+//  * G: eight lanes up to 26 unknowns, 16 for 35 to 50, a warp for 85 -- the
+//    triangle and the right-hand sides of 32 / G targets have to leave room for 8 to
+//    12 warps in 227 KB;
+//  * P: rows a lane keeps per block, whole blocks for the library's default lists
+//    (12, 20 and 36 neighbours in one; 40 in two of 20; 84 in three of 28); any
+//    other list runs ceil(k / P) blocks, 37 neighbours at degree 4 two of 36;
+//  * LS: four right-hand sides a pass where their 2 Q LS accumulators fit beside the
+//    columns (most bases of up to ten columns), else two;
+//  * MAXT: 384 threads (168 registers), 512 (128) for the smallest scalar bases, 256
+//    (255) for 35 columns and 85 unknowns; spills of up to about 300 bytes remain.
+// Neumann rows have the gradient-and-Laplacian set only: the Laplacian alone goes to
+// the shared-memory kernel.
 #define GMLS_SNE(KIND, D, DEG, L, G, P, LS, NEU, MAXT)                                                              \
   SneEntry {                                                                                                        \
     KIND, D, DEG, L, NEU, G, MAXT, SneLay<KIND, D, DEG, L, G, P, LS, NEU>::RHS,                                     \
