@@ -360,7 +360,7 @@ static cudaError_t launch_sne(gmls_ctx* ctx, const StencilJob& j, int deg, int k
 //    neighbours: 223 / 156 on one, 273 / 204 on 64, 271 / 891 on 900) and so are
 //    lists near the basis size (38: 500 / 343 on 2,048, 1084 / 1508 on 5,000);
 //  * shapes with only the shared-memory kernel beside it: 2,048 (2D scalar
-//    degree 4, 144 neighbours: 106 / 325);
+//    degree 4, 144 neighbours: 106 / 325), whatever the list;
 //  * lists shorter than 3/2 of the basis: some targets are ill-conditioned enough
 //    to be handed to the shared-memory kernel, a launch of 90 to 230 (2D scalar
 //    degree 4, 18 random neighbours: 281 / 170 on 2,048, 293 / 211 on 5,000,
@@ -372,17 +372,19 @@ static cudaError_t launch_sne(gmls_ctx* ctx, const StencilJob& j, int deg, int k
 //    2,048, 117 / 172 on 5,000);
 //  * lists above 400 leave few groups per SM (3D scalar degree 3, 500: 1030 / 913 on
 //    2,500);
-//  * otherwise 3,072 (2D scalar degree 4: 60 / 65 on 2,048, 71 / 108 on 5,000;
-//    3D degree-2 divergence-free, 64: 110 / 97 and 144 / 190).
+//  * otherwise 2,048 (2D scalar degree 4: 60 / 65 there, 71 / 108 on 5,000; 2D
+//    degree-2 divergence-free 49 / 50; the slowest 3D degree-2 divergence-free with
+//    64 neighbours: 110 / 97, 144 / 190 on 5,000).  Without the autotuner (the server)
+//    the kernel beside it is the one preferred at large sizes: 2D divergence-free
+//    degree 4, 97 / 196.
 static int64_t sne_min_targets(const StencilJob& j, int degree, int kmax, int nmax, bool reg) {
   const bool scalar = j.kind == GMLS_BASIS_SCALAR, staggered = j.kind == GMLS_BASIS_STAGGERED;
   const bool tight = 2 * kmax * j.nc < 3 * nmax;
   if (nmax >= 32) return scalar && tight ? 4096 : scalar && kmax > 128 ? 256 : 0;
   if (kmax > 400 && j.kind != GMLS_BASIS_DIVFREE) return 8192;
-  if (!reg) return 2048;
-  if (staggered) return kmax < 2 * nmax || degree == 4 ? 32768 : 4096;
-  if (tight && (scalar || j.dim == 2)) return 8192;
-  return 3072;
+  if (reg && staggered) return kmax < 2 * nmax || degree == 4 ? 32768 : 4096;
+  if (reg && tight && (scalar || j.dim == 2)) return 8192;
+  return 2048;
 }
 
 // Whether a call has the targets for the FP64 kernel of column-owning lanes.

@@ -92,11 +92,11 @@ def _same_bits(ctx, nid, basis, m, fns, precision, option, value, **kw):
 
 
 @pytest.mark.parametrize("dim,basis,m,fns,k,n,sne", [
-    (2, S, 3, [G, L], 20, 2500, False), (2, S, 3, [G, L], 20, 3600, True), (2, S, 4, [G, L], 18, 3600, False),
+    (2, S, 3, [G, L], 20, 1936, False), (2, S, 3, [G, L], 20, 2116, True), (2, S, 4, [G, L], 18, 3600, False),
     (2, S, 4, [G, L], 18, 8281, True), (2, S, 4, [G, L], 144, 2116, True), (2, S, 4, [G, L], 144, 1936, False),
     (2, T, 3, [G, L], 36, 3600, False), (2, T, 3, [G, L], 36, 4900, True), (2, T, 4, [G, L], 48, 4900, False),
     (3, T, 2, [G, L], 22, 4913, False), (3, F, 3, [V], 80, 343, True), (3, S, 4, [G, L], 84, 125, True),
-    (3, S, 4, [G, L], 140, 216, False), (3, S, 4, [G, L], 38, 2744, False), (2, F, 2, [V], 22, 2500, False)])
+    (3, S, 4, [G, L], 140, 216, False), (3, S, 4, [G, L], 38, 2744, False), (2, F, 2, [V], 22, 1936, False)])
 def test_fp32_choice_by_targets_and_list_length(ctx, dim, basis, m, fns, k, n, sne):
     nid = _cloud_list(ctx, dim, k, n)
     assert _same_bits(ctx, nid, basis, m, fns, gmls.FP32_REFINE, gmls.OPT_FORCE_VARIANT, -5) == sne
