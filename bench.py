@@ -103,7 +103,7 @@ def src_sha(*names):
 # DRAM bytes (read + write) per launch measured by ncu on the timed launch
 # (dram__bytes_read.sum + dram__bytes_write.sum, one pass), with the hash of
 # the kernel sources it was taken on; a different hash reports null
-SNE_TRAFFIC = {"bytes": 723164416 + 10174838016, "sha": "6fcfdf1d0f63de67",
+SNE_TRAFFIC = {"bytes": 722278400 + 10173070336, "sha": "3cd2f8e4f8c420f3",
                "sources": ("stencil_sne.cuh", "sne_d3.cu", "stencil_fast.cuh", "ff.cuh"),
                "command": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none --nvtx "
                           "--nvtx-include porous_step/ -k regex:stencil_sne -c 3 python bench.py --no-secondary "
