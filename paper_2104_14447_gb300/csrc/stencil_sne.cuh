@@ -56,7 +56,10 @@
 //    (s_f . s_lambda) / (s_f . s_f), f one more right-hand side.  A gradient row
 //    enters as its tangential part (the normal part n_c f / |n|^2 goes into beta
 //    alone), so rows along the normal, whose weights nearly vanish, lose nothing
-//    to the difference.
+//    to the difference.  The Laplacian row, on a one-sided target mostly beta s_f, is
+//    solved as lambda - beta_0 f with beta_0 from the FP32 factor for the same
+//    reason (without it its weights were 4 to 27 times further off than by
+//    elimination: 3D degree 2 1.1e-12, degree 3 6.1e-12).
 //  * Range: lambda carries eps^-1 or eps^-2 and the bounds above its squares, which
 //    leave FP32 already at eps = 1e-9 (a cloud of nanometres).  The systems are
 //    solved for lambda 2^(ORDER ee), 2^ee <= eps < 2^(ee + 1), ORDER the highest
@@ -1066,6 +1069,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
     // Laplacian (L = 1: the Laplacian alone; Neumann: then the normal derivative);
     // divergence-free: the vector Laplacian
     [[maybe_unused]] ff nv[D], in2;
+    [[maybe_unused]] float b0 = 0.0f;  // beta_0 of the Laplacian row, once known
     [[maybe_unused]] float fs = 1.0f;  // power of two that brings s_f (about |n| / eps, scaled) to order one
     if constexpr (NEU) {
       ff n2(0.f, 0.f);
@@ -1123,7 +1127,10 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
           for (int c = 0; c < D; ++c) v[c] = tg[c];
         }
         if (L != D) v[L == 1 ? 0 : D < LR ? D : 0] = lap * ie2;
-        if constexpr (NEU) v[L] = nd;
+        if constexpr (NEU) {
+          v[D] = v[D] - mul_f(nd, b0);
+          v[L] = nd;
+        }
       }
     };
     float w[LR][SN];
@@ -1334,6 +1341,20 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
       }
       // ---- 4. y = R^-1 R^-T w
       sne_solve<N, LR, G, SN, true>(R, ID, w, lane);
+      if constexpr (NEU)
+        if (step == 0) {  // s . s' = (R^-T lambda) . (R^-T lambda')
+          float num = 0.0f, den = 0.0f;
+#pragma unroll
+          for (int s = 0; s < SN; ++s)
+            if (s * G + lane < N) {
+              num = fmaf(w[D][s], w[L][s], num);
+              den = fmaf(w[L][s], w[L][s], den);
+            }
+          b0 = gsum<G>(num) / gsum<G>(den);
+          if (!(fabsf(b0) < 1e30f)) b0 = 0.0f;
+#pragma unroll
+          for (int s = 0; s < SN; ++s) w[D][s] = fmaf(-b0, w[L][s], w[D][s]);
+        }
       if (step == 0) {
         // accumulator constants of B^T s: |A e_q| |s|, |s| = |R^-T lambda|
 #pragma unroll
@@ -1512,7 +1533,7 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
           bt[l] = gsum<G>(pb[l].value()) * ff2;
           beta_ok = beta_ok && fabsf(bt[l].h) < 1e30f;  // (false for NaN)
           // (s = s_lambda - bt (fs s_f): beta = fs bt)
-          if (pending && lane == 0 && j.beta) j.beta[to * L + l] = to_double(l < D ? scale(bt[l]) + nv[l < D ? l : 0] * in2 : scale(bt[l]));
+          if (pending && lane == 0 && j.beta) j.beta[to * L + l] = to_double(l < D ? scale(bt[l]) + nv[l < D ? l : 0] * in2 : add_f(scale(bt[l]), b0));
         }
 #pragma unroll 1
         for (int q = lane; q < ke; q += G) {
