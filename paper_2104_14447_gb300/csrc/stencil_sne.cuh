@@ -782,9 +782,9 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
           mw += wt;
 #pragma unroll
           for (int c = 0; c < D; ++c) {
-            const float x = row_of(xi[c], e).h, wx = wt * x;
-            m1[c] += wx;
-            m2[c] = fmaf(wx, x, m2[c]);
+            const float x = row_of(xi[c], e).h;
+            m1[c] = fmaf(wt, x, m1[c]);
+            m2[c] = fmaf(wt * x, x, m2[c]);
           }
         }
 #pragma unroll
