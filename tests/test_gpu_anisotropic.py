@@ -78,11 +78,14 @@ def test_high_weight_powers_match_fp64(ctx, dim, basis, m, fns, k, power):
         ctx.release(h)
 
 
-@pytest.mark.parametrize("dim,m,k,axis", [(2, 2, 12, 70), (2, 3, 20, 70), (2, 4, 36, 70), (3, 2, 20, 17), (3, 3, 40, 17)])
-def test_neumann_laplacian_is_as_accurate_as_the_gradient(ctx, dim, m, k, axis):
+@pytest.mark.parametrize("dim,m,k,axis", [(2, 2, 12, 70), (3, 2, 20, 17), (2, 3, 20, 70), (2, 4, 36, 70), (3, 3, 40, 17),
+                                          (3, 4, 84, 14)])
+def test_neumann_rows_are_as_accurate_as_by_elimination(ctx, dim, m, k, axis):
     """On the one-sided targets of a box the constraint's share of the Laplacian
-    row is the larger part of it: solved without it, the row's error stays that of
-    the gradient (within 3/2; as a difference it was two to four times that)."""
+    row is the larger part of it.  Degree 2, whose systems are well conditioned: four
+    units of the kernel's sums (2^-43), or the shared-memory FP32 kernel's error,
+    which eliminates the constraint; degrees 3 and 4: the larger error of the two
+    functionals is no more than that kernel's (a quarter for the clouds' spread)."""
     x = inputs.jittered_grid(dim, axis, seed=3)
     n = x.shape[1]
     i = np.arange(n)
@@ -91,17 +94,17 @@ def test_neumann_laplacian_is_as_accurate_as_the_gradient(ctx, dim, m, k, axis):
     length = np.sqrt((nrm ** 2).sum(0))
     cid = ctx.cloud(x, normals=nrm / np.maximum(length, 1.0), bflags=(length > 0).astype(np.uint8))
     nid = ctx.neighbors(cid, k, 1.5)
-    ctx.set_option(gmls.OPT_FORCE_GENERIC, 1)
-    ref = ctx.stencils(nid, S, m, [G, L], precision=gmls.FP64, neumann=True)
-    ctx.set_option(gmls.OPT_FORCE_GENERIC, 0)
-    ctx.set_option(gmls.OPT_FORCE_VARIANT, -5)
-    sid = ctx.stencils(nid, S, m, [G, L], precision=gmls.FP32_REFINE, neumann=True)
-    ctx.set_option(gmls.OPT_FORCE_VARIANT, 0)
     bnd = torch.from_numpy(length > 0).cuda()
+    handles = []
+    for precision, option, value in ((gmls.FP64, gmls.OPT_FORCE_GENERIC, 1), (gmls.FP32_REFINE, gmls.OPT_FORCE_GENERIC, 1),
+                                     (gmls.FP32_REFINE, gmls.OPT_FORCE_VARIANT, -5)):
+        ctx.set_option(option, value)
+        handles.append(ctx.stencils(nid, S, m, [G, L], precision=precision, neumann=True))
+        ctx.set_option(option, 0)
     err = []
-    for fn in (G, L):
-        a, b = (ctx.weights(h, fn).view(n, -1)[bnd] for h in (sid, ref))
-        err.append(float((a - b).norm() / b.norm()))
-    assert err[1] <= 1.5 * err[0], err
-    for h in (sid, ref, nid, cid):
+    for h in handles[1:]:
+        pairs = [(ctx.weights(h, fn).view(n, -1)[bnd], ctx.weights(handles[0], fn).view(n, -1)[bnd]) for fn in (G, L)]
+        err.append(max(float((a - b).norm() / b.norm()) for a, b in pairs))
+    assert err[1] <= (max(4 * 2.0 ** -43, err[0]) if m == 2 else 1.25 * err[0]), err
+    for h in handles + [nid, cid]:
         ctx.release(h)
