@@ -1428,6 +1428,12 @@ __global__ void __launch_bounds__(MAXT, 1) stencil_sne_kernel(StencilJob j, cons
       }
       __syncwarp();
       float dmax = 0.0f, smax = 0.0f;
+      // a correction that is not finite (the maxima below drop NaN) hands the target on
+#pragma unroll
+      for (int l = 0; l < LR; ++l)
+#pragma unroll
+        for (int s = 0; s < SN; ++s)
+          if (s * G + lane < N && !(fabsf(w[l][s]) < 3e38f)) dmax = 3e38f;
       [[maybe_unused]] double others[L];
       [[maybe_unused]] Dot2 pb[LR];
       [[maybe_unused]] auto scale = [&](ff v) { return ff(v.h * fs, v.l * fs); };

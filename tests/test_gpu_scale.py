@@ -87,3 +87,17 @@ def test_beta_of_scaled_clouds(ctx, dim, m, k):
         out.append(beta)
     assert np.isfinite(out[0]).all() and (out[0] != 0).any()
     assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("basis,m,fns,k", [(S, 3, [G, L], 40), (S, 2, [L, G], 20), (F, 2, [V], 42)])
+def test_weights_beyond_the_fp32_range_go_to_other_kernels(ctx, basis, m, fns, k):
+    """At 1e14 the neighbour search of a 3D cloud stops short of the nearest
+    points (flagged), and targets far outside their lists have rows of 1e6 and more
+    times the usual size: a correction that is not finite does not count as
+    converged."""
+    nid, _ = _lists(ctx, 3, k, False, 1e14)
+    ctx.set_option(gmls.OPT_FORCE_VARIANT, -5)
+    sid = ctx.stencils(nid, basis, m, fns, precision=gmls.FP32_REFINE)
+    ctx.set_option(gmls.OPT_FORCE_VARIANT, 0)
+    for fn in fns:
+        assert bool(torch.isfinite(ctx.weights(sid, fn)).all())
