@@ -364,7 +364,8 @@ static cudaError_t launch_sne(gmls_ctx* ctx, const StencilJob& j, int deg, int k
 //  * lists shorter than 3/2 of the basis: some targets are ill-conditioned enough
 //    to be handed to the shared-memory kernel, a launch of 90 to 230 (2D scalar
 //    degree 4, 18 random neighbours: 281 / 170 on 2,048, 293 / 211 on 5,000,
-//    383 / 387 on 20,000);
+//    383 / 387 on 20,000; 2D divergence-free degree 3, 10: 150 / 68 on 2,048, 73 / 104 on
+//    5,000);
 //  * the staggered basis, whose columns have no constant, hands more over: below
 //    twice the basis and at degree 4 from 32,768 (degree 3, 17: 201 / 105 on
 //    5,000, 293 / 234 on 20,000, 622 / 818 on 80,000; degree 4, 48: 320 / 160,
@@ -383,7 +384,7 @@ static int64_t sne_min_targets(const StencilJob& j, int degree, int kmax, int nm
   if (nmax >= 32) return scalar && tight ? 4096 : scalar && kmax > 128 ? 256 : 0;
   if (kmax > 400 && j.kind != GMLS_BASIS_DIVFREE) return 8192;
   if (reg && staggered) return kmax < 2 * nmax || degree == 4 ? 32768 : 4096;
-  if (reg && tight && (scalar || j.dim == 2)) return 8192;
+  if (reg && tight && (scalar || j.dim == 2)) return scalar ? 8192 : 4096;
   return 2048;
 }
 
