@@ -460,7 +460,10 @@ gmls_status gmls_tune_info(gmls_ctx* ctx, int32_t index, int32_t* fields, float*
  * need to time anything (it never runs while capturing; uncached shapes then
  * use the heuristic choice).  Calls that must read device results on the host
  * (gmls_csr_size of radius-mode lists, exports to host) return GMLS_EBUSY or
- * fail during capture.  The graph handle is freed by gmls_release.
+ * fail during capture.  The graph handle is freed by gmls_release.  The graph's
+ * launches keep using the scratch they took from the arena: make objects that
+ * have to survive a gmls_graph_launch before gmls_capture_begin, or on another
+ * context.
  */
 gmls_status gmls_capture_begin(gmls_ctx* ctx);
 gmls_status gmls_capture_end(gmls_ctx* ctx, int64_t* graph_id);
